@@ -502,7 +502,7 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
   const int total = src.total();
 
   if (warp == 0 || warp == 2) {
-    if (lane == 0) {
+    if (tc::elect_one()) {
       // ------------------------------------------------ TMA producers
       // warp 0 copies the J tiles, warp 2 the S tiles of each stage (one
       // thread issues a TMA copy only every ~250 cycles); each arrives on the
@@ -634,7 +634,7 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
   } else if (warp == 1 && SPLIT && !lead) {
     // (second CTA of a split pair: the first CTA issues the pair's MMAs)
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (tc::elect_one()) {
       // ------------------------------------------------ MMA issuer
       uint32_t stage = 0, phase = 0;
       int it = 0;
@@ -1384,7 +1384,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   } while (0)
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (tc::elect_one()) {
       // ------------------------------------------------ TMA producer
       // the resident J tiles, once
       if (jres > 0) {
@@ -1473,7 +1473,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (tc::elect_one()) {
       // ------------------------------------------------ MMA issuer
       const uint32_t idesc = op_idesc(GN, FP8, P.f16);
       uint32_t stage = 0, phase = 0;
@@ -1881,7 +1881,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     const bool last = s + 1 == K;
     int wok = 1;
     if (warp == 0) {
-      if (lane == 0) {
+      if (tc::elect_one()) {
         for (int kt = 0; kt < nkt; ++kt) {
           const int kb = kt / P.planes;
           // descriptors of the tiles; K step k adds 32 bytes (2 in the >> 4 address field)
