@@ -1085,13 +1085,72 @@ struct TcResArgs {
   int nfull;           // k-blocks lying wholly below column n (pairs of them load as one box)
 };
 
+// Energies of restarts [b0, b0 + 32) of the step in slot ps, one warp: lane k
+// returns that of restart b0 + k (b0 + k < b1). The sums are track_kernel's:
+// lane l adds rows l, l + 32, ... starting from 0, then an xor tree over the
+// lanes. kTrackCols restarts go at a time, so a lane has that many row loads in
+// flight: the warp waits for one L2 round trip per 32 rows and kTrackCols
+// restarts. (With a lane per restart walking the rows, a slice of 8 restarts
+// over 32 rows took 24 us, and the CTA's next barrier arrival waits for it.)
+constexpr int kTrackCols = 8;
+template <bool INT_E>
+__device__ __forceinline__ double track_energies(const TcResArgs& R, int ps, int64_t b0, int64_t b1,
+                                                 int lane) {
+  const int64_t B = R.P.B;
+  double E = 0.0;
+  for (int c0 = 0; c0 < 32 && b0 + c0 < b1; c0 += kTrackCols) {
+    if (INT_E) {
+      long long q[kTrackCols], h[kTrackCols];
+#pragma unroll
+      for (int u = 0; u < kTrackCols; ++u) q[u] = h[u] = 0;
+      for (int r = lane; r < R.rows; r += 32) {
+        const int64_t o = (int64_t)r * B + b0 + c0;
+#pragma unroll
+        for (int u = 0; u < kTrackCols; ++u)
+          if (b0 + c0 + u < b1) q[u] += __ldcg(R.qpart[ps] + o + u);
+        if (R.P.has_h) {
+#pragma unroll
+          for (int u = 0; u < kTrackCols; ++u)
+            if (b0 + c0 + u < b1) h[u] += __ldcg(R.hpart[ps] + o + u);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kTrackCols; ++u) {
+        for (int w = 16; w; w >>= 1) q[u] += __shfl_xor_sync(0xffffffffu, q[u], w);
+        if (R.P.has_h)
+          for (int w = 16; w; w >>= 1) h[u] += __shfl_xor_sync(0xffffffffu, h[u], w);
+        if (lane == c0 + u) E = R.cq * (double)q[u] + R.chs * (double)h[u];
+      }
+    } else {
+      double e[kTrackCols];
+#pragma unroll
+      for (int u = 0; u < kTrackCols; ++u) e[u] = 0.0;
+      for (int r = lane; r < R.rows; r += 32) {
+        const int64_t o = (int64_t)r * B + b0 + c0;
+        float x[kTrackCols];
+#pragma unroll
+        for (int u = 0; u < kTrackCols; ++u)
+          x[u] = b0 + c0 + u < b1 ? __ldcg(R.epart[ps] + o + u) : 0.f;
+#pragma unroll
+        for (int u = 0; u < kTrackCols; ++u) e[u] += (double)x[u];
+      }
+#pragma unroll
+      for (int w = 16; w; w >>= 1)
+#pragma unroll
+        for (int u = 0; u < kTrackCols; ++u) e[u] += __shfl_xor_sync(0xffffffffu, e[u], w);
+#pragma unroll
+      for (int u = 0; u < kTrackCols; ++u)
+        if (lane == c0 + u) E = e[u];
+    }
+  }
+  return E;
+}
+
 // Best tracking of step t for restarts [b0, b1) by one warp, a lane per
-// restart, with the same sums as track_kernel (whose lane l adds rows l,
-// l + 32, ... starting from 0, then combines the lanes by an xor tree over
-// lane bits 4, 3, 2, 1, 0): here one lane forms the 32 lane sums and adds
-// them in that tree's order. The spins of the improved restarts are then
-// copied one restart at a time by the whole warp. With the convergence rule a
-// stopped restart is left alone, and steps t <= T feed the rule.
+// restart (energies as track_kernel forms them); the spins of the improved
+// restarts are then copied one restart at a time by the whole warp. With the
+// convergence rule a stopped restart is left alone, and steps t <= T feed the
+// rule.
 template <bool INT_E, bool FP8>
 __device__ __forceinline__ void track_warp(const TcResArgs& R, long long t, int64_t b0, int64_t b1,
                                            int lane) {
@@ -1102,32 +1161,10 @@ __device__ __forceinline__ void track_warp(const TcResArgs& R, long long t, int6
     const int64_t b = bb + lane;
     const bool ok = b < b1;
     bool improved = false;
+    const double best = ok ? R.best_E[b] : 0.0;
+    const double E = track_energies<INT_E>(R, ps, bb, b1, lane);
     const bool active = ok && (R.conv_step == nullptr || R.conv_step[b] == 0);
     if (active) {
-      const double best = R.best_E[b];
-      double E;
-      if (INT_E) {
-        long long q = 0, hs = 0;
-        for (int r = 0; r < R.rows; ++r) {
-          q += R.qpart[ps][(int64_t)r * P.B + b];
-          hs += R.hpart[ps][(int64_t)r * P.B + b];
-        }
-        E = R.cq * (double)q + R.chs * (double)hs;
-      } else {
-        double y[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          double lo = 0.0, hi = 0.0;  // the sums of lanes j and j + 16
-          for (int r = j; r < R.rows; r += 32) lo += (double)R.epart[ps][(int64_t)r * P.B + b];
-          for (int r = j + 16; r < R.rows; r += 32) hi += (double)R.epart[ps][(int64_t)r * P.B + b];
-          y[j] = lo + hi;
-        }
-#pragma unroll
-        for (int w = 8; w >= 1; w >>= 1)
-#pragma unroll
-          for (int j = 0; j < w; ++j) y[j] = y[j] + y[j + w];
-        E = y[0];
-      }
       improved = E < best;
       R.last_E[b] = E;
       if (improved) {
