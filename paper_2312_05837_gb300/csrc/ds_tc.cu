@@ -1088,16 +1088,43 @@ struct TcResArgs {
 // Energies of restarts [b0, b0 + 32) of the step in slot ps, one warp: lane k
 // returns that of restart b0 + k (b0 + k < b1). The sums are track_kernel's:
 // lane l adds rows l, l + 32, ... starting from 0, then an xor tree over the
-// lanes. kTrackCols restarts go at a time, so a lane has that many row loads in
-// flight: the warp waits for one L2 round trip per 32 rows and kTrackCols
-// restarts. (With a lane per restart walking the rows, a slice of 8 restarts
-// over 32 rows took 24 us, and the CTA's next barrier arrival waits for it.)
+// lanes. Below 32 rows (at most 7 row tiles, so slices of 10 to 32 restarts) a
+// lane forms its own restart's sum, all its row loads in flight at once; with
+// more rows and slices of at most 8 restarts the rows go to the lanes,
+// kTrackCols restarts at a time. Either way the warp waits for about one L2
+// round trip; walking the rows one by one took 24 us for 8 restarts x 32 rows,
+// and the CTA's next barrier arrival waits for it.
 constexpr int kTrackCols = 8;
 template <bool INT_E>
 __device__ __forceinline__ double track_energies(const TcResArgs& R, int ps, int64_t b0, int64_t b1,
                                                  int lane) {
   const int64_t B = R.P.B;
   double E = 0.0;
+  if (R.rows < 32) {
+    const bool ok = b0 + lane < b1;
+    if (INT_E) {
+      long long q = 0, h = 0;
+#pragma unroll 8
+      for (int r = 0; r < R.rows; ++r) {
+        const int64_t o = (int64_t)r * B + b0 + lane;
+        if (ok) q += __ldcg(R.qpart[ps] + o);
+        if (ok && R.P.has_h) h += __ldcg(R.hpart[ps] + o);
+      }
+      return R.cq * (double)q + R.chs * (double)h;
+    }
+    float x[32];
+#pragma unroll
+    for (int r = 0; r < 32; ++r)
+      x[r] = ok && r < R.rows ? __ldcg(R.epart[ps] + (int64_t)r * B + b0 + lane) : 0.f;
+    double y[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) y[j] = (double)x[j] + (double)x[j + 16];
+#pragma unroll
+    for (int w = 8; w >= 1; w >>= 1)
+#pragma unroll
+      for (int j = 0; j < w; ++j) y[j] = y[j] + y[j + w];
+    return y[0];
+  }
   for (int c0 = 0; c0 < 32 && b0 + c0 < b1; c0 += kTrackCols) {
     if (INT_E) {
       long long q[kTrackCols], h[kTrackCols];
