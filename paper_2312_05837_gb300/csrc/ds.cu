@@ -775,6 +775,7 @@ int ising::ds_create_impl(ising_ctx* ctx, const ising_instance* inst, const isin
     ISING_TRY(setup_field(ds));
     ISING_TRY(common_alloc(ds));
     ISING_TRY(init_state(ds));
+    if (ds->path == ISING_PATH_SPARSE) ISING_TRY(sparse_res_setup(ds));
     ISING_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return ISING_OK;
   }();
@@ -1015,6 +1016,10 @@ int ising::ds_advance(ising_ds* ds, int64_t todo) {
     if (ds->p.flags & ISING_DS_PROFILE) ds->kernel_launches += todo;
     return ISING_OK;
   }
+  if (ds->sres) {
+    if (ds->p.flags & ISING_DS_PROFILE) ds->kernel_launches += todo;
+    return sparse_res_run(ds, todo);
+  }
   int64_t s0 = 0;
   if (ds->path == ISING_PATH_SPARSE && !ds->tuned) ISING_TRY(autotune_sparse(ds, todo, &s0));
   if (ds->path == ISING_PATH_TC && !ds->tuned) ISING_TRY(autotune_dense(ds, todo, &s0));
@@ -1092,7 +1097,8 @@ extern "C" int ising_ds_run(ising_ds* ds, int64_t steps) {
   float ms = 0.f;
   cudaEventElapsedTime(&ms, e0, e1);
   ds->device_ms += ms;
-  if (ds->path == ISING_PATH_TC && tc_is_resident(ds) && (ds->p.flags & ISING_DS_PROFILE))
+  if (((ds->path == ISING_PATH_TC && tc_is_resident(ds)) || ds->sres) &&
+      (ds->p.flags & ISING_DS_PROFILE))
     ds->kernel_ms += ms;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -1369,6 +1375,7 @@ extern "C" int ising_ds_destroy(ising_ds* ds) {
   for (auto& e : ds->gev)
     if (e) cudaEventDestroy(e);
   tc_release(ds);
+  sparse_res_release(ds);
   delete ds;
   return ISING_OK;
 }

@@ -247,6 +247,8 @@ __device__ __forceinline__ void track_restart(const TrackArgs& A, long long t, i
 // spins x = sin(theta) (ISING_DS_RELAXED); energies then come from a
 // kModeEnergy pass on the rounded spins (dense paths) or from the rounded
 // spins gathered alongside (sparse path).
+struct SparseRes;  // resident sparse form (ds_sparse_res.cu)
+
 enum StepMode { kModeUpdate = 0, kModeEnergy = 1, kModeCoupling = 2, kModeRelaxed = 3 };
 
 }  // namespace ising
@@ -310,6 +312,7 @@ struct ising_ds {
   ising::DevMem sp_val;    // int8 or float values
   bool sp_int8 = false;
   int sp_q = 1;            // sparse slice width (x 128 restarts), chosen by the autotuner
+  ising::SparseRes* sres = nullptr;  // sparse path, resident form (null: a launch per step)
   bool tuned = false;
   // results
   bool finished = false;
@@ -338,6 +341,9 @@ int plain_setup(ising_ds* ds);
 int plain_step(ising_ds* ds, int mode, float* Gout);
 int sparse_setup(ising_ds* ds);
 int sparse_step(ising_ds* ds, int mode, float* Gout);
+int sparse_res_setup(ising_ds* ds);  // chooses the resident form (ds->sres) where it applies
+int sparse_res_run(ising_ds* ds, int64_t steps);  // queues `steps` steps, advances ds->t
+void sparse_res_release(ising_ds* ds);
 int tc_setup(ising_ds* ds);
 int tc_step(ising_ds* ds, int mode, float* Gout);
 int tc_error(ising_ds* ds);  // ISING_ETIMEOUT if a bounded wait gave up

@@ -1,14 +1,17 @@
 // K2s, resident form: domain selection (Sec. III-B) for CSR couplings whose
 // state fits the chip. Restarts are independent, so a CTA takes RB of them
 // and keeps everything they need in shared memory for a whole run of steps:
-// theta, m and v, the spins (one byte per site, bit r = restart r, two
-// buffers) and, when there is room, the couplings. A step then touches no
+// theta, m and v, the spins (two buffers: 16 bits per restart and site in the
+// form the sums take them, or one bit when that is all the room there is)
+// and, when there is room, the couplings. A step then touches no
 // global memory and waits for no other CTA: one launch runs all the steps
 // that the launch-per-step form takes two launches each for.
 //
-// What bounds it: instruction issue (about 50 per spin update and 7 per
-// coupling and pair of restarts) when RB n is large, the latency of one
-// gather, update and CTA barrier when it is small.
+// What bounds it: instruction issue when RB n is large (about 75 per spin
+// update, and 6 per coupling of a site whatever the restarts: the coupling's
+// word, its column and value, the neighbour's spins, a multiply-add per pair
+// of restarts), the latency of one gather, update and CTA barrier when it is
+// small.
 //
 // Couplings are stored as slices of 32 rows (the rows one warp takes
 // together), entry k of the slice's 32 rows side by side, padded with zero
@@ -38,6 +41,7 @@ struct SparseRes {
   int slices = 1;
   DevMem ell, off;
   int64_t entries = 0;  // coupling slots, padding included
+  bool pack = true;     // spins as 16 bits per restart and site, else as bits
   bool ell_smem = false;
   size_t smem = 0;
 };
@@ -49,10 +53,12 @@ struct SrArgs {
   int64_t B, Bp;
   int nt, rpb, kr, passes, nvb, slices;
   int64_t entries;
-  bool ell_smem;
-  const uint32_t* ell;  // V8: column | value << 16; else pairs (column, FP32 bits)
+  // shared-memory offsets in bytes (passed, not derived in the kernel: under
+  // register pressure the compiler would derive them again in every step)
+  int spins, buffer, part, off_at, ell_at;
+  const uint32_t* ell;  // V8: column | value << 24; else pairs (column, FP32 bits)
   const int* off;       // slice offsets in entries of 32 lanes
-  int64_t steps;
+  int steps;
   long long t0, T;
   StepConsts k;
   const float2* bias;
@@ -73,15 +79,16 @@ struct SrArgs {
   int* live32;
 };
 
-// Shared-memory layout (bytes), the same on both sides.
+// Shared-memory layout (bytes).
 struct SrLayout {
   size_t spins, part, off, ell, total;
-  __host__ __device__ SrLayout(int n, int rb, int nvb, int slices, int64_t entries, int ebytes,
-                               bool int_e, bool ell_smem) {
-    const size_t np = ((size_t)n + 15) / 16 * 16;
+  size_t buffer;  // bytes of one spin buffer
+  SrLayout(int n, int rb, int nvb, int slices, int64_t entries, int ebytes,
+                               bool int_e, bool pack, bool ell_smem) {
+    buffer = ((size_t)n * (pack ? 2 * rb : 1) + 15) / 16 * 16;
     spins = 12 * (size_t)n * rb;
     spins = (spins + 15) / 16 * 16;
-    part = spins + 2 * np;
+    part = spins + 2 * buffer;
     // INT: q and h, [2 slots][32 warps][rb]; else [2 slots][nvb][rb]
     const size_t pb = int_e ? (size_t)2 * 2 * 32 * rb * 4 : (size_t)2 * nvb * rb * 4;
     off = part + (pb + 15) / 16 * 16;
@@ -90,45 +97,110 @@ struct SrLayout {
   }
 };
 
+// Threads of a CTA at most: with 4 or 8 restarts a thread has enough to do at
+// half the warps, and needs the registers (64 spill).
+__host__ __device__ constexpr int sr_threads(int rb) { return rb >= 4 ? 512 : 1024; }
+
 // The row of thread `tid`, pass p, k-th row (or -1).
 __host__ __device__ __forceinline__ int sr_row(int n, int nt, int rpb, int tid, int p, int k) {
-  const int vw = p * nt + tid, w = vw & 7;
+  const int vw = p * nt + tid;
+  if (rpb == 8) return vw < n ? vw : -1;  // (one row per thread and pass)
+  const int w = vw & 7;
   const int64_t row = (int64_t)(vw >> 3) * rpb + w + 8 * k;
   return w + 8 * k < rpb && row < n ? (int)row : -1;
 }
 
-template <int RB, bool INT_E, bool V8>
-__global__ void __launch_bounds__(1024, 1) sparse_res_kernel(const SrArgs A) {
+// The spins of one site's RB restarts as 16-bit words, two to a register:
+// V8 (integer sums) +-1 as s_0 + 65536 s_1, so that adding value x word sums
+// both restarts at once; else BF16 +-1, each a shift or a mask away from FP32.
+template <int RB, bool V8>
+struct SpinWords {
+  static constexpr int W = (RB + 1) / 2;
+  uint32_t w[W];
+  __device__ __forceinline__ explicit SpinWords(uint32_t bits) {
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+      const uint32_t b0 = (bits >> (2 * k)) & 1u, b1 = (bits >> (2 * k + 1)) & 1u;
+      if (V8) w[k] = (2u * b0 - 1u) + (RB > 1 ? (2u * b1 - 1u) << 16 : 0u);
+      else w[k] = (b0 ? 0x3F80u : 0xBF80u) | (b1 ? 0x3F800000u : 0xBF800000u);
+    }
+  }
+  __device__ __forceinline__ SpinWords(const uint8_t* buf, int site) {
+    if constexpr (RB == 1) w[0] = V8 ? (uint32_t)(int)reinterpret_cast<const int16_t*>(buf)[site]
+                                     : reinterpret_cast<const uint16_t*>(buf)[site];
+    else if constexpr (RB == 2) w[0] = reinterpret_cast<const uint32_t*>(buf)[site];
+    else if constexpr (RB == 4) {
+      const uint2 x = reinterpret_cast<const uint2*>(buf)[site];
+      w[0] = x.x; w[1] = x.y;
+    } else {
+      const uint4 x = reinterpret_cast<const uint4*>(buf)[site];
+      w[0] = x.x; w[1] = x.y; w[2] = x.z; w[3] = x.w;
+    }
+  }
+  __device__ __forceinline__ void store(uint8_t* buf, int site) const {
+    if constexpr (RB == 1) reinterpret_cast<uint16_t*>(buf)[site] = (uint16_t)w[0];
+    else if constexpr (RB == 2) reinterpret_cast<uint32_t*>(buf)[site] = w[0];
+    else if constexpr (RB == 4) reinterpret_cast<uint2*>(buf)[site] = make_uint2(w[0], w[1]);
+    else reinterpret_cast<uint4*>(buf)[site] = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+};
+
+template <int RB, bool V8, bool PACK>
+__device__ __forceinline__ void store_spins(uint8_t* buf, int site, uint32_t bits) {
+  if constexpr (PACK) SpinWords<RB, V8>(bits).store(buf, site);
+  else buf[site] = (uint8_t)bits;
+}
+
+template <int RB, bool V8, bool PACK>
+__device__ __forceinline__ SpinWords<RB, V8> load_spins(const uint8_t* buf, int site) {
+  if constexpr (PACK) return SpinWords<RB, V8>(buf, site);
+  else return SpinWords<RB, V8>((uint32_t)buf[site]);
+}
+
+// ELLS: the couplings are in shared memory too (a pointer that may be either
+// costs 64-bit address arithmetic and generic loads per coupling).
+template <int RB, bool INT_E, bool V8, bool PACK, bool ELLS>
+__global__ void __launch_bounds__(sr_threads(RB), 1) sparse_res_kernel(const SrArgs A) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ uint32_t imp[2], alldone[2];
+  __shared__ float2 corr[2];  // Adam's bias corrections, slot s mod 2
+  // integer energies need no particular order: one row per thread and pass
+  const int kr = INT_E ? 1 : A.kr;
+  auto row_of = [&](int p, int k) {
+    if (!INT_E) return sr_row(A.n, A.nt, A.rpb, (int)threadIdx.x, p, k);
+    const int i = p * A.nt + (int)threadIdx.x;
+    return i < A.n ? i : -1;
+  };
   const int n = A.n, nt = A.nt, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const SrLayout L(n, RB, A.nvb, A.slices, A.entries, V8 ? 4 : 8, INT_E, A.ell_smem);
   float* sth = reinterpret_cast<float*>(smem);  // [RB][n]
-  float* smm = sth + (size_t)RB * n;
-  float* svv = smm + (size_t)RB * n;
-  const int np = (n + 15) / 16 * 16;
-  uint8_t* sp = smem + L.spins;  // [2][np]
-  int* pq = reinterpret_cast<int*>(smem + L.part);  // INT: [2][32][RB], then h
+  float* smm = sth + RB * n;
+  float* svv = smm + RB * n;
+  uint8_t* sp = smem + A.spins;  // two buffers
+  int* pq = reinterpret_cast<int*>(smem + A.part);  // INT: [2][32][RB], then h
   int* ph = pq + 2 * 32 * RB;
-  float* bs = reinterpret_cast<float*>(smem + L.part);  // else [2][nvb][RB]
-  int* soff = reinterpret_cast<int*>(smem + L.off);
-  const uint32_t* ell = A.ell_smem ? reinterpret_cast<const uint32_t*>(smem + L.ell) : A.ell;
+  float* bs = reinterpret_cast<float*>(smem + A.part);  // else [2][nvb][RB]
+  int* soff = reinterpret_cast<int*>(smem + A.off_at);
   const int64_t b0 = (int64_t)blockIdx.x * RB;
   const bool site = tid < nt;  // (the last warp tracks)
-  const int nidx = A.passes * A.kr;
+  const int nidx = A.passes * kr;
   const int nwarps = nt / 32;
 
   // the couplings, offsets and state of this CTA's restarts
   for (int e = tid; e <= A.slices; e += blockDim.x) soff[e] = A.off[e];
-  if (A.ell_smem) {
+  if (ELLS) {
     const uint4* src = reinterpret_cast<const uint4*>(A.ell);
-    uint4* dst = reinterpret_cast<uint4*>(smem + L.ell);
+    uint4* dst = reinterpret_cast<uint4*>(smem + A.ell_at);
     for (int64_t e = tid; e < A.entries * (V8 ? 4 : 8) / 16; e += blockDim.x) dst[e] = src[e];
   }
   if (tid < 2) alldone[tid] = 0, imp[tid] = 0;
+  // bit idx RB + r of these words: site idx of this thread, restart r. The
+  // spins of the step to come, of the last two steps, of the best step, and
+  // which sites the best ones were set for
+  uint32_t next_bits = 0, prev_bits = 0, prev2_bits = 0, best_bits = 0, any_bits = 0, rep = 0;
   if (site)
     for (int idx = 0; idx < nidx; ++idx) {
-      const int i = sr_row(n, nt, A.rpb, tid, idx / A.kr, idx % A.kr);
+      rep |= 1u << (idx * RB);
+      const int i = row_of(idx / kr, idx % kr);
       if (i < 0) continue;
       const int64_t g = (int64_t)i * A.Bp + b0;
       uint32_t byte = 0;
@@ -140,7 +212,8 @@ __global__ void __launch_bounds__(1024, 1) sparse_res_kernel(const SrArgs A) {
         svv[r * n + i] = A.v[g + r];
         byte |= (sin_nonneg(th) ? 1u : 0u) << r;
       }
-      sp[i] = (uint8_t)byte;
+      store_spins<RB, V8, PACK>(sp, i, byte);
+      next_bits |= byte << (idx * RB);
     }
   // tracking lane r: restart b0 + r
   const int64_t b = b0 + lane;
@@ -173,23 +246,34 @@ __global__ void __launch_bounds__(1024, 1) sparse_res_kernel(const SrArgs A) {
   if (tid == 0) alldone[0] = 0;
 
   // Energies and bests of step index e, by the tracking warp.
-  auto track = [&](int64_t e) {
-    const int slot = (int)(e & 1);
+  auto track = [&](int e) {
+    const int slot = e & 1;
     const long long t = A.t0 + e + 1;
     double E = 0.0;
+    if (INT_E) {
 #pragma unroll
-    for (int r = 0; r < RB; ++r) {
-      if (INT_E) {
+      for (int r = 0; r < RB; ++r) {
         const int q = __reduce_add_sync(0xffffffffu, lane < nwarps ? pq[(slot * 32 + lane) * RB + r] : 0);
         int h = 0;
         if (A.hf) h = __reduce_add_sync(0xffffffffu, lane < nwarps ? ph[(slot * 32 + lane) * RB + r] : 0);
-        if (lane == r) E = A.cq * (double)(long long)q + A.chs * (double)(long long)h;
-      } else {
-        double x = 0.0;
-        for (int c = lane; c < A.nvb; c += 32) x += (double)bs[(slot * A.nvb + c) * RB + r];
-        for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane == r) E = x;
+        if (lane == r) E = A.cq * (double)q + A.chs * (double)h;
       }
+    } else {
+      // (the restarts' FP64 chains side by side: one after another they were
+      // the longest part of a step)
+      double x[RB];
+#pragma unroll
+      for (int r = 0; r < RB; ++r) x[r] = 0.0;
+      for (int c = lane; c < A.nvb; c += 32)
+#pragma unroll
+        for (int r = 0; r < RB; ++r) x[r] += (double)bs[(slot * A.nvb + c) * RB + r];
+#pragma unroll
+      for (int o = 16; o; o >>= 1)
+#pragma unroll
+        for (int r = 0; r < RB; ++r) x[r] += __shfl_xor_sync(0xffffffffu, x[r], o);
+#pragma unroll
+      for (int r = 0; r < RB; ++r)
+        if (lane == r) E = x[r];
     }
     bool better = false;
     if (!stopped) {
@@ -223,29 +307,29 @@ __global__ void __launch_bounds__(1024, 1) sparse_res_kernel(const SrArgs A) {
     }
   };
 
-  // bit idx RB + r of these words: site idx of this thread, restart r; the
-  // spins consumed at the last two steps, the best ones, which have changed
-  uint32_t prev_bits = 0, prev2_bits = 0, best_bits = 0, any_bits = 0, rep = 0;
-  for (int idx = 0; idx < nidx; ++idx) rep |= 1u << (idx * RB);
-  float2 bc = A.bias[A.t0 + 1];
-  int64_t s = 0;
+  const float2* bias = A.bias + A.t0 + 1;  // of step index 0
+  if (!site && lane == 0) corr[0] = bias[0];
+  __syncthreads();
+  int s = 0;
   bool early = false;
   if (!retired)
     for (; s < A.steps; ++s) {
-      const int cur = (int)(s & 1);
-      const uint8_t* spc = sp + cur * np;
-      uint8_t* spn = sp + (cur ^ 1) * np;
+      const int cur = s & 1;
+      const uint8_t* spc = sp + cur * A.buffer;
+      uint8_t* spn = sp + (cur ^ 1) * A.buffer;
       if (!site) {
+        if (lane == 0 && s + 1 < A.steps) corr[cur ^ 1] = bias[s + 1];
         if (s >= 1) track(s - 1);
       } else {
-        const float2 bcs = bc;
-        if (s + 1 < A.steps) bc = A.bias[A.t0 + s + 2];
+        const float2 bcs = corr[cur];
         if (s >= 2) {
           const uint32_t mk = imp[cur] * rep;  // the bests of step s - 2
           best_bits = (best_bits & ~mk) | (prev2_bits & mk);
           any_bits |= mk;
         }
-        uint32_t cur_bits = 0;
+        prev2_bits = prev_bits;
+        prev_bits = next_bits;
+        next_bits = 0;
         int eq[RB], eh[RB];
 #pragma unroll
         for (int r = 0; r < RB; ++r) eq[r] = eh[r] = 0;
@@ -253,56 +337,53 @@ __global__ void __launch_bounds__(1024, 1) sparse_res_kernel(const SrArgs A) {
           float ee[RB];
 #pragma unroll
           for (int r = 0; r < RB; ++r) ee[r] = 0.f;
-          for (int k = 0; k < A.kr; ++k) {
-            const int idx = p * A.kr + k;
-            const int i = sr_row(n, nt, A.rpb, tid, p, k);
+          for (int k = 0; k < kr; ++k) {
+            const int idx = p * kr + k;
+            const int i = row_of(p, k);
             const int sl = idx * nwarps + warp;
-            const int e0 = soff[sl], e1 = soff[sl + 1];
+            const int cnt = soff[sl + 1] - soff[sl], e0 = soff[sl] * 32 + lane;
             float G[RB];
             int Gi[RB];
             if constexpr (V8) {
-              // sums over the neighbours with spin +1, two restarts per word
-              // (each half's sum fits 16 bits), and over all neighbours
               constexpr int W = (RB + 1) / 2;
-              int P[W], V = 0;
+              int P[W];
 #pragma unroll
               for (int w = 0; w < W; ++w) P[w] = 0;
+              const uint32_t* en = (ELLS ? reinterpret_cast<const uint32_t*>(smem + A.ell_at) : A.ell) + e0;
 #pragma unroll 4
-              for (int e = e0; e < e1; ++e) {
-                const uint32_t en = ell[e * 32 + lane];
-                const int val = (int)(en << 8) >> 24;
-                const uint32_t y = spc[en & 0xFFFFu];
-                V += val;
+              for (int e = 0; e < cnt; ++e, en += 32) {
+                const uint32_t x = *en;
+                const int val = (int)x >> 24;
+                const SpinWords<RB, V8> y = load_spins<RB, V8, PACK>(spc, (int)(x & 0xFFFFFFu));
 #pragma unroll
-                for (int w = 0; w < W; ++w) {
-                  const uint32_t u = RB == 1 ? y : ((y >> (2 * w)) & 1u) | ((y << (15 - 2 * w)) & 0x10000u);
-                  P[w] += (int)u * val;
-                }
+                for (int w = 0; w < W; ++w) P[w] += (int)y.w[w] * val;
               }
 #pragma unroll
               for (int r = 0; r < RB; ++r) {
                 const int lo = (int)(int16_t)(P[r / 2] & 0xFFFF);
-                const int pr = RB == 1 ? P[0] : ((r & 1) ? (P[r / 2] - lo) >> 16 : lo);
-                Gi[r] = 2 * pr - V;
+                Gi[r] = RB == 1 ? P[0] : ((r & 1) ? (P[r / 2] - lo) >> 16 : lo);
                 G[r] = (float)Gi[r];
               }
             } else {
 #pragma unroll
               for (int r = 0; r < RB; ++r) G[r] = 0.f;
-#pragma unroll 2
-              for (int e = e0; e < e1; ++e) {
-                const uint2 en = reinterpret_cast<const uint2*>(ell)[e * 32 + lane];
-                const uint32_t y = ~(uint32_t)spc[en.x];
+              const uint2* en = reinterpret_cast<const uint2*>(
+                  ELLS ? reinterpret_cast<const uint32_t*>(smem + A.ell_at) : A.ell) + e0;
+#pragma unroll 4
+              for (int e = 0; e < cnt; ++e, en += 32) {
+                const uint2 x = *en;
+                const SpinWords<RB, V8> y = load_spins<RB, V8, PACK>(spc, (int)x.x);
+                const float J = __uint_as_float(x.y);
+                // G + J s, one rounding, as G + (s > 0 ? J : -J)
 #pragma unroll
                 for (int r = 0; r < RB; ++r)
-                  G[r] += __uint_as_float(en.y ^ ((y << (31 - r)) & 0x80000000u));
+                  G[r] = fmaf(J, __uint_as_float((r & 1) ? y.w[r / 2] & 0xFFFF0000u : y.w[r / 2] << 16), G[r]);
               }
 #pragma unroll
               for (int r = 0; r < RB; ++r) Gi[r] = INT_E ? __float2int_rn(G[r]) : 0;
             }
             if (i < 0) continue;
-            const uint32_t own = spc[i];
-            cur_bits |= own << (idx * RB);
+            const uint32_t own = prev_bits >> (idx * RB);
             const float h = A.hf ? __ldg(A.hf + i) : 0.f;
             const int hi = INT_E && A.hf ? __ldg(A.hint + i) : 0;
             uint32_t byte = 0;
@@ -325,7 +406,8 @@ __global__ void __launch_bounds__(1024, 1) sparse_res_kernel(const SrArgs A) {
               svv[r * n + i] = v;
               byte |= (sin_nonneg(th) ? 1u : 0u) << r;
             }
-            spn[i] = (uint8_t)byte;
+            store_spins<RB, V8, PACK>(spn, i, byte);
+            next_bits |= byte << (idx * RB);
           }
           if (!INT_E) {
             // the 8 rows' sums of a block in warp order
@@ -350,8 +432,6 @@ __global__ void __launch_bounds__(1024, 1) sparse_res_kernel(const SrArgs A) {
             }
           }
         }
-        prev2_bits = prev_bits;
-        prev_bits = cur_bits;
       }
       __syncthreads();
       // (alldone[cur] is written at step s only, by the tracking of s - 1)
@@ -362,7 +442,7 @@ __global__ void __launch_bounds__(1024, 1) sparse_res_kernel(const SrArgs A) {
     }
   // the last step's energies (none when every restart stopped before it),
   // then the bests of the last two steps
-  const int64_t last = early ? s : s - 1;  // index of the last step computed
+  const int last = early ? s : s - 1;  // index of the last step computed
   if (!retired) {
     if (!site && !early) track(last);
     __syncthreads();
@@ -379,10 +459,9 @@ __global__ void __launch_bounds__(1024, 1) sparse_res_kernel(const SrArgs A) {
       }
     }
   }
-  const uint8_t* spf = sp + (retired ? 0 : (int)((last + 1) & 1)) * np;
   if (site)
     for (int idx = 0; idx < nidx; ++idx) {
-      const int i = sr_row(n, nt, A.rpb, tid, idx / A.kr, idx % A.kr);
+      const int i = row_of(idx / kr, idx % kr);
       if (i < 0) continue;
       const int64_t g = (int64_t)i * A.Bp + b0;
 #pragma unroll
@@ -395,7 +474,8 @@ __global__ void __launch_bounds__(1024, 1) sparse_res_kernel(const SrArgs A) {
         if ((any_bits >> (idx * RB + r)) & 1u)
           A.best_s[(b0 + r) * A.bs_ld + i] = ((best_bits >> (idx * RB + r)) & 1u) ? 1 : -1;
       }
-      atomicOr(&A.bits_out[(int64_t)i * (A.Bp / 32) + (b0 >> 5)], (uint32_t)spf[i] << (b0 & 31));
+      const uint32_t bits = (next_bits >> (idx * RB)) & ((1u << RB) - 1u);
+      atomicOr(&A.bits_out[(int64_t)i * (A.Bp / 32) + (b0 >> 5)], bits << (b0 & 31));
     }
   if (mine) {
     A.best_E[b] = bE;
@@ -498,7 +578,7 @@ __global__ void sr_fill_kernel(int n, int nt, int rpb, int kr, int slices, bool 
     const uint32_t c = k < d ? (uint32_t)col[a + k] : 0u;
     if (v8) {
       const uint32_t x = k < d ? (uint8_t)static_cast<const int8_t*>(val)[a + k] : 0u;
-      ell[e] = c | (x << 16);
+      ell[e] = c | (x << 24);
     } else {
       const float x = k < d ? static_cast<const float*>(val)[a + k] : 0.f;
       reinterpret_cast<uint2*>(ell)[e] = make_uint2(c, __float_as_uint(x));
@@ -506,9 +586,10 @@ __global__ void sr_fill_kernel(int n, int nt, int rpb, int kr, int slices, bool 
   }
 }
 
-template <int RB, bool INT_E, bool V8>
+template <int RB, bool INT_E, bool V8, bool PACK>
 int sr_launch(ising_ds* ds, const SparseRes* R, const SrArgs& a) {
-  auto kern = sparse_res_kernel<RB, INT_E, V8>;
+  auto kern = R->ell_smem ? sparse_res_kernel<RB, INT_E, V8, PACK, true>
+                          : sparse_res_kernel<RB, INT_E, V8, PACK, false>;
   ISING_CUDA(ds->ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)(ds->ctx->smem_optin - 1024)));
   kern<<<(unsigned)((ds->B + RB - 1) / RB), R->nt + 32, R->smem, ds->ctx->stream>>>(a);
@@ -516,16 +597,23 @@ int sr_launch(ising_ds* ds, const SparseRes* R, const SrArgs& a) {
   return ISING_OK;
 }
 
-template <int RB>
+template <int RB, bool PACK>
 int sr_launch_rb(ising_ds* ds, const SparseRes* R, const SrArgs& a) {
-  if (ds->int_energy) return ds->sp_int8 ? sr_launch<RB, true, true>(ds, R, a) : sr_launch<RB, true, false>(ds, R, a);
-  return ds->sp_int8 ? sr_launch<RB, false, true>(ds, R, a) : sr_launch<RB, false, false>(ds, R, a);
+  if (ds->int_energy)
+    return ds->sp_int8 ? sr_launch<RB, true, true, PACK>(ds, R, a) : sr_launch<RB, true, false, PACK>(ds, R, a);
+  return ds->sp_int8 ? sr_launch<RB, false, true, PACK>(ds, R, a) : sr_launch<RB, false, false, PACK>(ds, R, a);
+}
+
+template <int RB>
+int sr_launch_pack(ising_ds* ds, const SparseRes* R, const SrArgs& a) {
+  return R->pack ? sr_launch_rb<RB, true>(ds, R, a) : sr_launch_rb<RB, false>(ds, R, a);
 }
 
 }  // namespace
 
 // Whether the session runs this form, and its operands. It does when the
-// state of RB restarts fits a CTA's shared memory (n RB up to about 18000),
+// state of RB restarts fits a CTA's shared memory (n RB up to about 18000,
+// 14000 with 16-bit spins),
 // with RB the least of 1, 2, 4, 8 that gives every SM at most one CTA, or 8
 // (several waves of CTAs then): the launch-per-step form costs at least two
 // launches and an L2 round trip per coupling however small the instance.
@@ -545,6 +633,9 @@ int sparse_res_setup(ising_ds* ds) {
   R.rb = 8;
   for (int c : {4, 2, 1})
     if (ceil_div_i(ds->B, c) <= ctx->sm_count) R.rb = c;
+  // a CTA runs until its slowest restart stops: under the convergence rule
+  // fewer of them per CTA retire sooner
+  if (ds->conv.p) R.rb = std::min(R.rb, 2);
   if (ds->int_energy) {
     R.rpb = 8;
     R.nvb = ceil_div_i(n, 8);
@@ -556,15 +647,16 @@ int sparse_res_setup(ising_ds* ds) {
   }
   R.kr = ceil_div_i(R.rpb, 8);
   const int vw = R.nvb * 8;
-  constexpr int kMaxSite = 992;
-  R.passes = ceil_div_i(vw, kMaxSite);
+  R.passes = ceil_div_i(vw, sr_threads(R.rb) - 32);
   R.nt = (ceil_div_i(vw, R.passes) + 31) / 32 * 32;
   if (R.passes * R.kr * R.rb > 32) return ISING_OK;  // (a bit per site and restart of a thread)
   R.slices = R.passes * R.kr * (R.nt / 32);
   const size_t limit = ctx->smem_optin - 1024;
   const int ebytes = v8 ? 4 : 8;
-  if (SrLayout((int)n, R.rb, R.nvb, R.slices, 0, ebytes, ds->int_energy, false).total > limit)
-    return ISING_OK;
+  auto bytes = [&](bool pack, bool ell) {
+    return SrLayout((int)n, R.rb, R.nvb, R.slices, R.entries, ebytes, ds->int_energy, pack, ell).total;
+  };
+  if (bytes(false, false) > limit) return ISING_OK;
   ISING_TRY(dev_alloc(ctx, R.off, ((size_t)R.slices + 2) * 4));
   ISING_CUDA(ctx, cudaMemsetAsync(R.off.p, 0, R.off.bytes, ctx->stream));
   const int g = ceil_div_i((int64_t)R.slices * 32, 256);
@@ -585,10 +677,9 @@ int sparse_res_setup(ising_ds* ds) {
                                              I.rowptr.as<int32_t>(), I.indices.as<int32_t>(),
                                              ds->sp_val.p, R.off.as<int>(), R.ell.as<uint32_t>());
   ISING_CUDA(ctx, cudaGetLastError());
-  R.smem = SrLayout((int)n, R.rb, R.nvb, R.slices, R.entries, ebytes, ds->int_energy, true).total;
-  R.ell_smem = R.smem <= limit;
-  if (!R.ell_smem)
-    R.smem = SrLayout((int)n, R.rb, R.nvb, R.slices, R.entries, ebytes, ds->int_energy, false).total;
+  R.pack = bytes(true, false) <= limit;
+  R.ell_smem = bytes(R.pack, true) <= limit;
+  R.smem = bytes(R.pack, R.ell_smem);
   ds->sres = new SparseRes(std::move(R));
   return ISING_OK;
 }
@@ -608,8 +699,14 @@ int sparse_res_run(ising_ds* ds, int64_t steps) {
   a.nvb = R->nvb;
   a.slices = R->slices;
   a.entries = R->entries;
-  a.ell_smem = R->ell_smem;
   a.ell = R->ell.as<uint32_t>();
+  const SrLayout L((int)ds->n, R->rb, R->nvb, R->slices, R->entries, ds->sp_int8 ? 4 : 8,
+                   ds->int_energy, R->pack, R->ell_smem);
+  a.spins = (int)L.spins;
+  a.buffer = (int)L.buffer;
+  a.part = (int)L.part;
+  a.off_at = (int)L.off;
+  a.ell_at = (int)L.ell;
   a.off = R->off.as<int>();
   a.T = ds->T;
   a.k = ds->k;
@@ -638,13 +735,13 @@ int sparse_res_run(ising_ds* ds, int64_t steps) {
     DevMem& out = ds->spins[(ds->t + k + 1) % 3];
     ISING_CUDA(ctx, cudaMemsetAsync(out.p, 0, out.bytes, ctx->stream));
     a.bits_out = out.as<uint32_t>();
-    a.steps = k;
+    a.steps = (int)k;
     a.t0 = ds->t;
     switch (R->rb) {
-      case 1: ISING_TRY(sr_launch_rb<1>(ds, R, a)); break;
-      case 2: ISING_TRY(sr_launch_rb<2>(ds, R, a)); break;
-      case 4: ISING_TRY(sr_launch_rb<4>(ds, R, a)); break;
-      default: ISING_TRY(sr_launch_rb<8>(ds, R, a)); break;
+      case 1: ISING_TRY(sr_launch_pack<1>(ds, R, a)); break;
+      case 2: ISING_TRY(sr_launch_pack<2>(ds, R, a)); break;
+      case 4: ISING_TRY(sr_launch_pack<4>(ds, R, a)); break;
+      default: ISING_TRY(sr_launch_pack<8>(ds, R, a)); break;
     }
     if (conv) {
       sr_work_kernel<<<ceil_div_i(ds->B, 128), 128, 0, ctx->stream>>>(

@@ -174,7 +174,8 @@ int start_request(ising_server* srv, Request* r, double ms[3]) {
     // convergence rule or the relaxed product: each CTA holds all of J and
     // its restarts, no grid barrier), which runs a whole chunk in one launch
     const bool small = red.n <= 128 && !(p.flags & (ISING_DS_CONVERGE | ISING_DS_RELAXED));
-    if (!small) p.flags |= ISING_DS_STREAMING;
+    // (the sparse resident form has no grid barrier either)
+    if (!small && red.layout == ISING_LAYOUT_DENSE) p.flags |= ISING_DS_STREAMING;
     ISING_TRY(ds_create_impl(ctx, &red, &p, &r->ds, false));
   }
   ISING_CUDA(ctx, cudaEventCreateWithFlags(&r->ev, cudaEventDisableTiming));
