@@ -166,6 +166,10 @@ struct ResLayout {
   static constexpr uint32_t kB = GN * kRowBytes;
   static constexpr uint32_t kStage = kKps * (kA + kB);
   static constexpr int kMaxStages = 8;
+  // epilogue warps: four per part of the group's columns, at least one chunk each
+  static constexpr int kParts = GN >= 32 ? 4 : GN / 8;
+  static constexpr int kCols = GN / kParts;
+  static constexpr int kEpi = 4 * kParts;
 };
 
 // Sum over the 32 lanes of each of 8 columns; afterwards lanes l, l^1, l^2,
@@ -1246,7 +1250,7 @@ __device__ __forceinline__ void resident_chunks(const TcResArgs& R, const EpiLan
                                                 bool last, uint64_t* acc_empty, uint32_t& sbits,
                                                 int sh) {
   const TcArgs& P = R.P;
-  constexpr int kCols = GN / 4;
+  constexpr int kCols = ResLayout<GN>::kCols;
   const uint32_t t_th = Gr.t_acc + GN, t_m = Gr.t_acc + 2 * GN, t_v = Gr.t_acc + 3 * GN;
   void* Sout = R.spins[(t + 1) % 3];
   const int ps = (int)(t % 2);
@@ -1369,7 +1373,8 @@ __device__ __forceinline__ void resident_chunks(const TcResArgs& R, const EpiLan
   }
 }
 
-template <int GN, bool INT_E, bool FP8>
+// GR: restart groups per CTA (1 or 2).
+template <int GN, int GR, bool INT_E, bool FP8>
 __global__ void __launch_bounds__(kThreads, 1)
     tc_resident_kernel(const __grid_constant__ CUtensorMap tmA0,
                        const __grid_constant__ CUtensorMap tmA1,
@@ -1388,8 +1393,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int STAGES = R.nst;
   const int jres = R.jres;
   constexpr int kBK = FP8 ? 128 : 64;
-  constexpr uint32_t kTmemCols = 8 * GN;  // per group: accumulator, theta, m, v
-  constexpr int kCols = GN / 4;           // columns of a group per epilogue warp
+  constexpr uint32_t kTmemCols = 4 * GN * GR;  // per group: accumulator, theta, m, v
+  constexpr int kCols = Lay::kCols;            // columns of a group per epilogue warp
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -1411,10 +1416,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc::mbar_init(&full[s], 1);
       tc::mbar_init(&empty[s], 1);
     }
-    for (int g = 0; g < 2; ++g) {
+    for (int g = 0; g < GR; ++g) {
       tc::mbar_init(&acc_full[g], 1);
-      tc::mbar_init(&acc_empty[g], kEpiWarps);
-      tc::mbar_init(&step_done[g], kEpiWarps);
+      tc::mbar_init(&acc_empty[g], Lay::kEpi);
+      tc::mbar_init(&step_done[g], Lay::kEpi);
       tc::mbar_init(&go[g], 1);
     }
     tc::mbar_init(drain, 1);
@@ -1431,10 +1436,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem_base = *tmem_slot;
   const long long t0 = P.counters[0];
   const int64_t K = R.steps;
-  const int64_t NP = 2 * K;  // phases: step s of group g is phase 2 s + g
+  const int64_t NP = GR * K;  // phases: step s of group g is phase GR s + g
   const int mt = blockIdx.x % P.mtiles;
   const int64_t m0 = (int64_t)mt * kBM;
-  const int64_t n0 = (int64_t)(blockIdx.x / P.mtiles) * (2 * GN);  // first restart of the CTA
+  const int64_t n0 = (int64_t)(blockIdx.x / P.mtiles) * (GR * GN);  // first restart of the CTA
   const int nkt = P.nk * P.planes;
   // role timeline of one step of group 0 (profiling): 0 producer starts the
   // step, 1 last TMA issued, 2 last MMA committed, 3 controller finished
@@ -1465,8 +1470,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       int issued = 0;
       bool ok = true;
       for (int64_t p = 0; p < NP && ok; ++p) {
-        const int64_t s = p >> 1;
-        const int g = (int)(p & 1);
+        const int64_t s = p / GR;
+        const int g = (int)(p % GR);
         const long long t = t0 + s + 1;
         const int slot = (int)(t % 3);
         const CUtensorMap* mb = slot == 0 ? &tmB0 : (slot == 1 ? &tmB1 : &tmB2);
@@ -1543,8 +1548,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t stage = 0, phase = 0;
       bool ok = jres == 0 || tc::mbar_wait(jfull, 0, abort_flag, kWaitCycles);
       for (int64_t p = 0; p < NP && ok; ++p) {
-        const int64_t s = p >> 1;
-        const int g = (int)(p & 1);
+        const int64_t s = p / GR;
+        const int g = (int)(p % GR);
         const uint32_t d = tmem_base + (uint32_t)(g * 4 * GN);
         if (!tc::mbar_wait(&acc_empty[g], (uint32_t)((s & 1) ^ 1), abort_flag, kWaitCycles)) {
           ok = false;
@@ -1589,7 +1594,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         atomicExch(R.gabort, 1);
       }
     }
-  } else if (warp == 2 || warp == 3) {
+  } else if (warp == 2 || (GR == 2 && warp == 3)) {
     // ------------------------------------------------ column-barrier controller
     // of group g = warp - 2, and its best tracking: the CTAs of one restart
     // group's column (all m-tiles of the same restarts) exchange spins;
@@ -1598,7 +1603,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // the barrier of step s + 1, which any overwrite of the step's partials
     // and spins (at step s + 2) has to wait for.
     const int g = warp - 2;
-    unsigned int* colbar = R.gbar + 32 * (2 * (blockIdx.x / P.mtiles) + g);
+    unsigned int* colbar = R.gbar + 32 * (GR * (blockIdx.x / P.mtiles) + g);
     const int64_t gs = n0 + g * GN;
     const int64_t ge = gs + GN < P.B ? gs + GN : P.B;
     const int64_t tb0 = gs + (int64_t)mt * R.slice;
@@ -1636,10 +1641,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       track_warp<INT_E, FP8>(R, t0 + s + 1, tb0, tb1, lane);
       if (lane == 0) ISING_RTRACE(3, s, g);
     }
-  } else {
+  } else if (warp >= 4 && warp < 4 + Lay::kEpi) {
     // ------------------------------------------------ epilogue
     const int q = warp & 3;
-    const int part = (warp - 4) >> 2;  // which quarter of a group's columns
+    const int part = (warp - 4) >> 2;  // which part of a group's columns
     const int64_t i = m0 + 32 * q + lane;
     const bool row_ok = i < P.n;
     const float h = row_ok ? P.hf[i] : 0.f;
@@ -1664,7 +1669,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // state of this warp's columns into tensor memory, and the signs of theta
     // (bit g kCols + c for column c of group g)
     uint32_t sbits = 0;
-    for (int g = 0; g < 2; ++g) {
+    for (int g = 0; g < GR; ++g) {
       const EpiGroup Gr = group(g);
 #pragma unroll 1
       for (int c0 = 0; c0 < kCols; c0 += kChunk) {
@@ -1688,8 +1693,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc::tmem_wait_st();
     bool ok = true;
     for (int64_t p = 0; p < NP && ok; ++p) {
-      const int64_t s = p >> 1;
-      const int g = (int)(p & 1);
+      const int64_t s = p / GR;
+      const int g = (int)(p % GR);
       const long long t = t0 + s + 1;
       const float2 bc = P.bias[t];  // loaded ahead of the wait, off the critical path
       if (!tc::mbar_wait(&acc_full[g], (uint32_t)(s & 1), abort_flag, kWaitCycles)) {
@@ -2141,7 +2146,9 @@ struct TcState {
   bool resident = false;  // one tile per CTA, state kept in tensor memory
   DevMem gsync;           // abort word + per-column barrier counters
   int emode = 0;          // resident epilogue's integer energy mode (0 F2I, 1 offset, 2 packed)
-  int gn = 64;            // resident forms: restarts per group (two per CTA; small form: one)
+  int gn = 64;            // resident forms: restarts per group
+  int gr = 2;             // resident form: groups per CTA
+  int res_grid = 0;       // resident form: CTAs
   bool small = false;     // small form (n <= 128): all of J per CTA, spins kept on chip
   size_t small_bytes = 0;
   int small_grid = 0;     // small form: CTAs (one per block of gn restarts)
@@ -2286,37 +2293,41 @@ int launch_relaxed(ising_ds* ds, TcState* st, const TcArgs& a, const CUtensorMap
 
 }  // namespace
 
-template <int GN, bool INT_E, bool FP8>
+template <int GN, int GR, bool INT_E, bool FP8>
 int resident_attr(ising_ctx* ctx, size_t smem, int* blocks_per_sm) {
-  auto kern = tc_resident_kernel<GN, INT_E, FP8>;
+  auto kern = tc_resident_kernel<GN, GR, INT_E, FP8>;
   ISING_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   ISING_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, kThreads, smem));
   return ISING_OK;
 }
 
-template <int GN, bool INT_E, bool FP8>
+template <int GN, int GR, bool INT_E, bool FP8>
 int resident_launch(ising_ds* ds, TcState* st, const TcResArgs& ra) {
-  auto kern = tc_resident_kernel<GN, INT_E, FP8>;
+  auto kern = tc_resident_kernel<GN, GR, INT_E, FP8>;
   void* args[] = {&st->A[0],  &st->A[1],  &st->A[2],  &st->Bg[0], &st->Bg[1], &st->Bg[2],
                   &st->J2[0], &st->J2[1], &st->J2[2], &st->S2[0], &st->S2[1], &st->S2[2],
                   const_cast<TcResArgs*>(&ra)};
-  ISING_CUDA(ds->ctx, cudaLaunchCooperativeKernel((const void*)kern, dim3(st->grid), dim3(kThreads),
+  ISING_CUDA(ds->ctx, cudaLaunchCooperativeKernel((const void*)kern, dim3(st->res_grid), dim3(kThreads),
                                                   args, st->res_bytes, ds->ctx->stream));
   return ISING_OK;
 }
 
-template <int GN>
+template <int GN, int GR>
 int resident_attr_bn(ising_ds* ds, bool fp8, size_t smem, int* nb) {
   if (ds->int_energy)
-    return fp8 ? resident_attr<GN, true, true>(ds->ctx, smem, nb) : resident_attr<GN, true, false>(ds->ctx, smem, nb);
-  return fp8 ? resident_attr<GN, false, true>(ds->ctx, smem, nb) : resident_attr<GN, false, false>(ds->ctx, smem, nb);
+    return fp8 ? resident_attr<GN, GR, true, true>(ds->ctx, smem, nb)
+               : resident_attr<GN, GR, true, false>(ds->ctx, smem, nb);
+  return fp8 ? resident_attr<GN, GR, false, true>(ds->ctx, smem, nb)
+             : resident_attr<GN, GR, false, false>(ds->ctx, smem, nb);
 }
 
-template <int BN>
+template <int GN, int GR>
 int resident_launch_bn(ising_ds* ds, TcState* st, const TcResArgs& ra) {
   if (ds->int_energy)
-    return st->fp8 ? resident_launch<BN, true, true>(ds, st, ra) : resident_launch<BN, true, false>(ds, st, ra);
-  return st->fp8 ? resident_launch<BN, false, true>(ds, st, ra) : resident_launch<BN, false, false>(ds, st, ra);
+    return st->fp8 ? resident_launch<GN, GR, true, true>(ds, st, ra)
+                   : resident_launch<GN, GR, true, false>(ds, st, ra);
+  return st->fp8 ? resident_launch<GN, GR, false, true>(ds, st, ra)
+                 : resident_launch<GN, GR, false, false>(ds, st, ra);
 }
 
 template <int BN, bool INT_E, bool FP8>
@@ -2340,7 +2351,7 @@ int small_launch_bn(ising_ds* ds, TcState* st, const TcSmallArgs& a) {
 // Abort word, then one arrival counter per restart group of each column, 128
 // bytes apart.
 static size_t gsync_bytes(const ising_ds* ds, const TcState* st) {
-  return (size_t)(1 + 2 * ceil_div_i(ds->B, st->BN)) * 128;
+  return (size_t)(1 + st->gr * ceil_div_i(ds->B, st->gr * st->gn)) * 128;
 }
 
 int tc_setup(ising_ds* ds) {
@@ -2479,39 +2490,48 @@ int tc_setup(ising_ds* ds) {
     }
   }
   if (!st->resident && !(ds->p.flags & ISING_DS_STREAMING) && !ds->relaxed()) {
-    const int gn = ds->B > 64 ? 64 : 32;
-    const int tiles = ceil_div_i(ds->n, kBM) * ceil_div_i(ds->B, 2 * gn);
-    // shared memory: resident J tiles (as many as leave room for 4 stages of 2 k-blocks),
-    // then the stages, then the barrier block
-    const int64_t kA = (int64_t)kBM * kRowBytes, kStage = 2 * (kA + (int64_t)gn * kRowBytes);
-    const int64_t region = ((int64_t)ctx->smem_optin - 1024 - 512) / 1024 * 1024;
-    const int nkt = ceil_div_i(ds->n, st->fp8 ? 128 : 64) * ds->planes;
-    const int jres = (int)std::min<int64_t>(nkt, std::max<int64_t>(0, (region - 4 * kStage) / kA));
-    const int nst = (int)std::min<int64_t>(8, (region - jres * kA) / kStage);
-    int nb = 0;
-    if (nst >= 2) {
-      const size_t bytes = (size_t)region + 512 + 1024;
-      ISING_TRY(gn == 64 ? resident_attr_bn<64>(ds, st->fp8, bytes, &nb)
-                         : resident_attr_bn<32>(ds, st->fp8, bytes, &nb));
-      if (nb >= 1 && tiles <= nb * ctx->sm_count) {
-        st->resident = true;
-        st->BN = 2 * gn;
-        st->gn = gn;
-        st->grid = tiles;
-        st->jres = jres;
-        st->nst = nst;
-        st->bars = (uint32_t)region;
-        st->res_bytes = bytes;
+    // one group of 16, 32 or 64 restarts per CTA, the fewest that give every
+    // tile its own SM (a step's epilogue, bound by instruction issue, then
+    // spreads over the most SMs), else two groups of 64 in turn
+    const int mt = ceil_div_i(ds->n, kBM);
+    auto fits = [&](int width) { return (int64_t)mt * ceil_div_i(ds->B, width) <= ctx->sm_count; };
+    int gn = 0, gr = 1;
+    for (int c : {16, 32, 64})
+      if (!gn && fits(c)) gn = c;
+    if (!gn && fits(128)) gn = 64, gr = 2;
+    if (gn) {
+      // shared memory: resident J tiles (as many as leave room for 4 stages of
+      // 2 k-blocks), then the stages, then the barrier block
+      const int64_t kA = (int64_t)kBM * kRowBytes, kStage = 2 * (kA + (int64_t)gn * kRowBytes);
+      const int64_t region = ((int64_t)ctx->smem_optin - 1024 - 512) / 1024 * 1024;
+      const int nkt = ceil_div_i(ds->n, st->fp8 ? 128 : 64) * ds->planes;
+      const int jres = (int)std::min<int64_t>(nkt, std::max<int64_t>(0, (region - 4 * kStage) / kA));
+      const int nst = (int)std::min<int64_t>(8, (region - jres * kA) / kStage);
+      int nb = 0;
+      if (nst >= 2) {
+        const size_t bytes = (size_t)region + 512 + 1024;
+        if (gr == 2) ISING_TRY((resident_attr_bn<64, 2>(ds, st->fp8, bytes, &nb)));
+        else if (gn == 64) ISING_TRY((resident_attr_bn<64, 1>(ds, st->fp8, bytes, &nb)));
+        else if (gn == 32) ISING_TRY((resident_attr_bn<32, 1>(ds, st->fp8, bytes, &nb)));
+        else ISING_TRY((resident_attr_bn<16, 1>(ds, st->fp8, bytes, &nb)));
+        if (nb >= 1) {
+          st->resident = true;
+          st->gn = gn;
+          st->gr = gr;
+          st->res_grid = mt * ceil_div_i(ds->B, gr * gn);
+          st->BN = ds->B <= 64 ? 64 : 128;  // (the final evaluation's tiles)
+          st->jres = jres;
+          st->nst = nst;
+          st->bars = (uint32_t)region;
+          st->res_bytes = bytes;
+        }
       }
     }
   }
-  if (st->resident && !st->small) {
-    ISING_TRY(dev_alloc(ctx, st->gsync, gsync_bytes(ds, st)));
-  } else {
-    // streaming launches (and, in the small form, the final evaluation)
-    const int tiles = ceil_div_i(ds->n, kBM) * ceil_div_i(ds->B, st->BN);
-    st->grid = std::max(1, std::min(tiles, ctx->sm_count));
-  }
+  if (st->resident && !st->small) ISING_TRY(dev_alloc(ctx, st->gsync, gsync_bytes(ds, st)));
+  // streaming launches (in the resident forms, the final evaluation)
+  const int tiles = ceil_div_i(ds->n, kBM) * ceil_div_i(ds->B, st->BN);
+  st->grid = std::max(1, std::min(tiles, ctx->sm_count));
   return ISING_OK;
 }
 
@@ -2591,7 +2611,7 @@ int tc_run(ising_ds* ds, int mode, float* Gout) {
     a.trk = track_args(ds);
   }
   if (ds->p.flags & ISING_DS_PROFILE) {
-    if (!st->trace.p) ISING_TRY(dev_alloc(ds->ctx, st->trace, (size_t)st->grid * 8 * 8));
+    if (!st->trace.p) ISING_TRY(dev_alloc(ds->ctx, st->trace, (size_t)std::max(st->grid, st->res_grid) * 8 * 8));
     a.trace = st->trace.as<unsigned long long>();
   }
   const CUtensorMap& mS = st->B[t % 3];
@@ -2716,7 +2736,7 @@ int tc_run_resident(ising_ds* ds, int64_t steps) {
   a.live32 = nullptr;  // the resident forms do not retire restarts
   a.work = nullptr;
   if (ds->p.flags & ISING_DS_PROFILE) {
-    if (!st->trace.p) ISING_TRY(dev_alloc(ds->ctx, st->trace, (size_t)st->grid * 8 * 8));
+    if (!st->trace.p) ISING_TRY(dev_alloc(ds->ctx, st->trace, (size_t)std::max(st->grid, st->res_grid) * 8 * 8));
     a.trace = st->trace.as<unsigned long long>();
   }
   r.steps = steps;
@@ -2747,7 +2767,10 @@ int tc_run_resident(ising_ds* ds, int64_t steps) {
   r.nst = st->nst;
   r.bars = st->bars;
   r.nfull = st->nfull;
-  return st->gn == 64 ? resident_launch_bn<64>(ds, st, r) : resident_launch_bn<32>(ds, st, r);
+  if (st->gr == 2) return resident_launch_bn<64, 2>(ds, st, r);
+  return st->gn == 64 ? resident_launch_bn<64, 1>(ds, st, r)
+                      : (st->gn == 32 ? resident_launch_bn<32, 1>(ds, st, r)
+                                      : resident_launch_bn<16, 1>(ds, st, r));
 }
 
 int tc_error(ising_ds* ds) {
@@ -2764,11 +2787,12 @@ int tc_trace(ising_ds* ds, uint64_t* out, int64_t cap, int64_t* count) {
   auto st = static_cast<TcState*>(ds->tc);
   *count = 0;
   if (!st || !st->trace.p) return ISING_OK;
-  const int64_t n = std::min<int64_t>(cap, (int64_t)st->grid * 8);
+  const int64_t total = (int64_t)(st->resident && !st->small ? st->res_grid : st->grid) * 8;
+  const int64_t n = std::min<int64_t>(cap, total);
   if (n > 0)
     ISING_CUDA(ds->ctx, cudaMemcpyAsync(out, st->trace.p, n * 8, cudaMemcpyDeviceToHost, ds->ctx->stream));
   ISING_CUDA(ds->ctx, cudaStreamSynchronize(ds->ctx->stream));
-  *count = (int64_t)st->grid * 8;
+  *count = total;
   return ISING_OK;
 }
 
