@@ -155,17 +155,20 @@ struct TcLayout {
   static constexpr uint32_t kTmemCols = 2 * BN <= 128 ? 128 : (2 * BN <= 256 ? 256 : 512);
 };
 
-// Resident form: shared memory holds the first `jres` J tiles of the CTA's
-// rows for the whole run (J does not change between steps), then `nst`
-// stages of a J tile and the S tile of one restart group (GN); the later J
-// tiles stream through the stages. Sizes are chosen at launch (TcResArgs).
+// Resident form: the operands of a step come in units of two J tiles: two
+// k-blocks of the one plane, or both planes of one k-block, with the S tiles
+// of those k-blocks (two, or the one that both planes share). Shared memory
+// holds the J tiles of the first `ru` units for the whole run (J does not
+// change between steps), a ring of `nj` unit slots through which the later
+// ones stream and a ring of `ns` unit slots for S. J waits for nothing but its
+// ring, so its copies run ahead of the column barrier. Sizes are chosen at
+// launch (TcResArgs).
 template <int GN>
 struct ResLayout {
-  static constexpr int kKps = 2;  // k-blocks per stage: [J tiles][S tiles]
   static constexpr uint32_t kA = kBM * kRowBytes;
   static constexpr uint32_t kB = GN * kRowBytes;
-  static constexpr uint32_t kStage = kKps * (kA + kB);
-  static constexpr int kMaxStages = 8;
+  static constexpr uint32_t kJ = 2 * kA;  // J tiles of a unit
+  static constexpr int kMaxSlots = 16;
   // epilogue warps: four per part of the group's columns, at least one chunk each
   static constexpr int kParts = GN >= 32 ? 4 : GN / 8;
   static constexpr int kCols = GN / kParts;
@@ -1082,8 +1085,8 @@ struct TcResArgs {
   double* conv_init;
   long long* conv_step;
   unsigned long long* conv_count;
-  int jres;            // J tiles (k-blocks) kept in shared memory for the whole run
-  int nst;             // pipeline stages after them
+  int ru;              // units whose J tiles stay in shared memory for the whole run
+  int nj, ns;          // slots of the J and the S ring after them
   uint32_t bars;       // shared-memory offset of the barrier block
   int slice;           // restarts of a group tracked per CTA of its column
   int nfull;           // k-blocks lying wholly below column n (pairs of them load as one box)
@@ -1390,19 +1393,23 @@ __global__ void __launch_bounds__(kThreads, 1)
                        const __grid_constant__ CUtensorMap tmS2_2, const TcResArgs R) {
   const TcArgs& P = R.P;
   using Lay = ResLayout<GN>;
-  const int STAGES = R.nst;
-  const int jres = R.jres;
+  const int ru = R.ru, nj = R.nj, ns = R.ns;
   constexpr int kBK = FP8 ? 128 : 64;
   constexpr uint32_t kTmemCols = 4 * GN * GR;  // per group: accumulator, theta, m, v
   constexpr int kCols = Lay::kCols;            // columns of a group per epilogue warp
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  uint8_t* stages = smem + (size_t)jres * Lay::kA;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + R.bars);
-  uint64_t* empty = full + Lay::kMaxStages;
-  uint64_t* jfull = empty + Lay::kMaxStages;  // the resident J tiles have landed
-  uint64_t* acc_full = jfull + 1;       // [2], one per restart group
+  const bool two = P.planes == 2;
+  const uint32_t kS = two ? Lay::kB : 2 * Lay::kB;  // S tiles of a unit
+  uint8_t* jring = smem + (uint32_t)ru * Lay::kJ;
+  uint8_t* sring = jring + (uint32_t)nj * Lay::kJ;
+  uint64_t* sfull = reinterpret_cast<uint64_t*>(smem + R.bars);
+  uint64_t* sempty = sfull + Lay::kMaxSlots;
+  uint64_t* jfull = sempty + Lay::kMaxSlots;
+  uint64_t* jempty = jfull + Lay::kMaxSlots;
+  uint64_t* rfull = jempty + Lay::kMaxSlots;  // the resident J tiles have landed
+  uint64_t* acc_full = rfull + 1;       // [2], one per restart group
   uint64_t* acc_empty = acc_full + 2;   // [2]
   uint64_t* step_done = acc_empty + 2;  // [2]
   uint64_t* go = step_done + 2;         // [2]
@@ -1412,9 +1419,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      tc::mbar_init(&full[s], 1);
-      tc::mbar_init(&empty[s], 1);
+    for (int s = 0; s < Lay::kMaxSlots; ++s) {
+      tc::mbar_init(&sfull[s], 1);
+      tc::mbar_init(&sempty[s], 1);
+      tc::mbar_init(&jfull[s], 1);
+      tc::mbar_init(&jempty[s], 1);
     }
     for (int g = 0; g < GR; ++g) {
       tc::mbar_init(&acc_full[g], 1);
@@ -1423,7 +1432,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc::mbar_init(&go[g], 1);
     }
     tc::mbar_init(drain, 1);
-    tc::mbar_init(jfull, 1);
+    tc::mbar_init(rfull, 1);
     *abort_flag = 0;
     tc::fence_barrier_init();
   }
@@ -1441,6 +1450,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int64_t m0 = (int64_t)mt * kBM;
   const int64_t n0 = (int64_t)(blockIdx.x / P.mtiles) * (GR * GN);  // first restart of the CTA
   const int nkt = P.nk * P.planes;
+  const int units = (nkt + 1) / 2;
   // role timeline of one step of group 0 (profiling): 0 producer starts the
   // step, 1 last TMA issued, 2 last MMA committed, 3 controller finished
   // tracking the step, 4 epilogue has the accumulator, 5 epilogue done,
@@ -1452,91 +1462,92 @@ __global__ void __launch_bounds__(kThreads, 1)
       P.trace[(size_t)blockIdx.x * 8 + (slot)] = now_ns();                          \
   } while (0)
 
+  // tile t of unit u: k-block and plane
+  auto block_of = [&](int u, int t) { return two ? u : 2 * u + t; };
+  auto map_a = [&](int plane) { return plane == 0 ? &tmA0 : &tmA1; };
   if (warp == 0) {
     if (tc::elect_one()) {
       // ------------------------------------------------ TMA producer
-      // the resident J tiles, once
-      if (jres > 0) {
-        tc::mbar_expect_tx(jfull, (uint32_t)jres * Lay::kA);
-        // (unit kt of a step is plane kt % planes of k-block kt / planes: the
-        // planes k-block by k-block, the order of every form)
-        for (int kt = 0; kt < jres; ++kt) {
-          const int plane = kt % P.planes, kb = kt / P.planes;
-          const CUtensorMap* ma = plane == 0 ? &tmA0 : (plane == 1 ? &tmA1 : &tmA2);
-          tc::tma_load_2d(smem + (size_t)kt * Lay::kA, ma, jfull, kb * kBK, (int)m0);
+      auto copy_j = [&](uint8_t* dst, uint64_t* bar, int u) {
+        const int cnt = nkt - 2 * u < 2 ? nkt - 2 * u : 2;
+        tc::mbar_expect_tx(bar, (uint32_t)cnt * Lay::kA);
+        if (!two && 2 * u + 1 < R.nfull) {
+          // two whole k-blocks of the plane: one box
+          tc::tma_load_3d(dst, &tmJ2_0, bar, 0, (int)m0, 2 * u);
+        } else {
+          for (int t = 0; t < cnt; ++t)
+            tc::tma_load_2d(dst + t * Lay::kA, map_a(two ? t : 0), bar, block_of(u, t) * kBK, (int)m0);
         }
+      };
+      for (int u = 0; u < ru; ++u) {
+        if (u == 0) tc::mbar_expect_tx(rfull, (uint32_t)(min(2 * ru, nkt)) * Lay::kA);
+        const int cnt = nkt - 2 * u < 2 ? nkt - 2 * u : 2;
+        for (int t = 0; t < cnt; ++t)
+          tc::tma_load_2d(smem + (uint32_t)u * Lay::kJ + t * Lay::kA, map_a(two ? t : 0), rfull,
+                          block_of(u, t) * kBK, (int)m0);
       }
-      uint32_t stage = 0, phase = 0;
-      int issued = 0;
+      uint32_t js = 0, jphase = 0, ss = 0, sphase = 0;
+      int64_t jissued = 0, sissued = 0;
+      const int su = units - ru;  // streamed units of a phase
       bool ok = true;
+      // streamed unit j of the phase, when its slot is free
+      auto next_j = [&](int j) {
+        if (!tc::mbar_wait(&jempty[js], jphase ^ 1, abort_flag, kWaitCycles)) return false;
+        copy_j(jring + js * Lay::kJ, &jfull[js], ru + j);
+        ++jissued;
+        if (++js == (uint32_t)nj) { js = 0; jphase ^= 1; }
+        return true;
+      };
       for (int64_t p = 0; p < NP && ok; ++p) {
         const int64_t s = p / GR;
         const int g = (int)(p % GR);
         const long long t = t0 + s + 1;
-        const int slot = (int)(t % 3);
-        const CUtensorMap* mb = slot == 0 ? &tmB0 : (slot == 1 ? &tmB1 : &tmB2);
-        const CUtensorMap* mb2 = slot == 0 ? &tmS2_0 : (slot == 1 ? &tmS2_1 : &tmS2_2);
+        const int sl = (int)(t % 3);
+        const CUtensorMap* mb = sl == 0 ? &tmB0 : (sl == 1 ? &tmB1 : &tmB2);
+        const CUtensorMap* mb2 = sl == 0 ? &tmS2_0 : (sl == 1 ? &tmS2_1 : &tmS2_2);
         const int nb = (int)(n0 + g * GN);
-        if (s > 0) {
+        // J as far as its ring goes, then S of the units in order, each J unit
+        // once S is a ring ahead of the unit whose slot it waits for
+        int j = 0;
+        for (; j < nj && j < su && ok; ++j) ok = next_j(j);
+        if (s > 0 && ok) {
           // S_t of the group exists once every CTA of its column is through step t - 1
-          if (!tc::mbar_wait(&go[g], (uint32_t)((s - 1) & 1), abort_flag, kWaitCycles)) {
-            ok = false;
-            break;
-          }
+          ok = tc::mbar_wait(&go[g], (uint32_t)((s - 1) & 1), abort_flag, kWaitCycles);
           tc::fence_proxy_async_global();
         }
         ISING_RTRACE(0, s, g);
-        for (int kt0 = 0; kt0 < nkt; kt0 += Lay::kKps) {
-          if (!tc::mbar_wait(&empty[stage], phase ^ 1, abort_flag, kWaitCycles)) {
+        for (int u = 0; u < units && ok; ++u) {
+          if (!tc::mbar_wait(&sempty[ss], sphase ^ 1, abort_flag, kWaitCycles)) {
             ok = false;
             break;
           }
-          uint8_t* sa = stages + (size_t)stage * Lay::kStage;
-          uint32_t bytes = 0;
-#pragma unroll
-          for (int u = 0; u < Lay::kKps; ++u) {
-            const int kt = kt0 + u;
-            if (kt < nkt) bytes += kt < jres ? Lay::kB : Lay::kA + Lay::kB;
-          }
-          tc::mbar_expect_tx(&full[stage], bytes);
-          const int plane0 = kt0 % P.planes, kb0 = kt0 / P.planes;
-          if (P.planes == 1 && kb0 + 1 < R.nfull) {
-            // two whole k-blocks of one plane: one box each for J and S (the
-            // issue of a TMA instruction, not its bytes, paces this thread)
-            if (kt0 >= jres) {
-              const CUtensorMap* ma = plane0 == 0 ? &tmJ2_0 : (plane0 == 1 ? &tmJ2_1 : &tmJ2_2);
-              tc::tma_load_3d(sa, ma, &full[stage], 0, (int)m0, kb0);
-            } else if (kt0 + 1 >= jres) {
-              const CUtensorMap* ma = plane0 == 0 ? &tmA0 : (plane0 == 1 ? &tmA1 : &tmA2);
-              tc::tma_load_2d(sa + Lay::kA, ma, &full[stage], (kb0 + 1) * kBK, (int)m0);
-            }
-            tc::tma_load_3d(sa + Lay::kKps * Lay::kA, mb2, &full[stage], 0, nb, kb0);
+          uint8_t* dst = sring + ss * kS;
+          const int cnt = two ? 1 : (nkt - 2 * u < 2 ? nkt - 2 * u : 2);
+          tc::mbar_expect_tx(&sfull[ss], (uint32_t)cnt * Lay::kB);
+          if (!two && 2 * u + 1 < R.nfull) {
+            tc::tma_load_3d(dst, mb2, &sfull[ss], 0, nb, 2 * u);
           } else {
-#pragma unroll
-            for (int u = 0; u < Lay::kKps; ++u) {
-              const int kt = kt0 + u;
-              if (kt >= nkt) break;
-              const int plane = kt % P.planes, kb = kt / P.planes;
-              if (kt >= jres) {
-                const CUtensorMap* ma = plane == 0 ? &tmA0 : (plane == 1 ? &tmA1 : &tmA2);
-                tc::tma_load_2d(sa + u * Lay::kA, ma, &full[stage], kb * kBK, (int)m0);
-              }
-              tc::tma_load_2d(sa + Lay::kKps * Lay::kA + u * Lay::kB, mb, &full[stage], kb * kBK, nb);
-            }
+            for (int i = 0; i < cnt; ++i)
+              tc::tma_load_2d(dst + i * Lay::kB, mb, &sfull[ss], block_of(u, i) * kBK, nb);
           }
-          ++issued;
-          if (++stage == (uint32_t)STAGES) { stage = 0; phase ^= 1; }
+          ++sissued;
+          if (++ss == (uint32_t)ns) { ss = 0; sphase ^= 1; }
+          while (ok && j < su && ru + j - nj + ns - 1 <= u) ok = next_j(j++);
         }
+        while (ok && j < su) ok = next_j(j++);
         ISING_RTRACE(1, s, g);
       }
       if (!ok) {
-        int back = issued < STAGES ? issued : STAGES;
-        uint32_t s2 = stage, ph = phase;
-        for (int q = 0; q < back; ++q) {
-          if (s2 == 0) { s2 = STAGES - 1; ph ^= 1; } else { --s2; }
-          tc::mbar_wait(&full[s2], ph, nullptr, kWaitCycles / 8);
+        // let the copies already issued land before the CTA exits
+        for (int64_t q = jissued < nj ? jissued : nj; q > 0; --q) {
+          if (js == 0) { js = nj - 1; jphase ^= 1; } else { --js; }
+          tc::mbar_wait(&jfull[js], jphase, nullptr, kWaitCycles / 8);
         }
-        if (jres > 0) tc::mbar_wait(jfull, 0, nullptr, kWaitCycles / 8);
+        for (int64_t q = sissued < ns ? sissued : ns; q > 0; --q) {
+          if (ss == 0) { ss = ns - 1; sphase ^= 1; } else { --ss; }
+          tc::mbar_wait(&sfull[ss], sphase, nullptr, kWaitCycles / 8);
+        }
+        if (ru > 0) tc::mbar_wait(rfull, 0, nullptr, kWaitCycles / 8);
         atomicExch(P.err, 1);
         atomicExch(R.gabort, 1);
       }
@@ -1545,8 +1556,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (tc::elect_one()) {
       // ------------------------------------------------ MMA issuer
       const uint32_t idesc = op_idesc(GN, FP8, P.f16);
-      uint32_t stage = 0, phase = 0;
-      bool ok = jres == 0 || tc::mbar_wait(jfull, 0, abort_flag, kWaitCycles);
+      uint32_t js = 0, jphase = 0, ss = 0, sphase = 0;
+      bool ok = ru == 0 || tc::mbar_wait(rfull, 0, abort_flag, kWaitCycles);
       for (int64_t p = 0; p < NP && ok; ++p) {
         const int64_t s = p / GR;
         const int g = (int)(p % GR);
@@ -1556,33 +1567,35 @@ __global__ void __launch_bounds__(kThreads, 1)
           break;
         }
         tc::fence_after_sync();
-        for (int kt0 = 0; kt0 < nkt; kt0 += Lay::kKps) {
-          if (!tc::mbar_wait(&full[stage], phase, abort_flag, kWaitCycles)) {
+        for (int u = 0; u < units; ++u) {
+          const bool streamed = u >= ru;
+          if ((streamed && !tc::mbar_wait(&jfull[js], jphase, abort_flag, kWaitCycles)) ||
+              !tc::mbar_wait(&sfull[ss], sphase, abort_flag, kWaitCycles)) {
             ok = false;
             break;
           }
           tc::fence_after_sync();
-          const uint32_t sb = tc::smem_u32(stages + (size_t)stage * Lay::kStage);
+          const uint32_t a0 = tc::smem_u32(streamed ? jring + js * Lay::kJ : smem + (uint32_t)u * Lay::kJ);
+          const uint32_t b0 = tc::smem_u32(sring + ss * kS);
 #pragma unroll
-          for (int u = 0; u < Lay::kKps; ++u) {
-            const int kt = kt0 + u;
-            if (kt >= nkt) break;
-            const uint32_t a0 = kt < jres ? tc::smem_u32(smem + (size_t)kt * Lay::kA) : sb + u * Lay::kA;
+          for (int t = 0; t < 2; ++t) {
+            if (2 * u + t >= nkt) break;
             // descriptors of the tiles; K step k adds 32 bytes (2 in the >> 4 address field)
-            const uint64_t da = tc::desc_k_sw128(a0);
-            const uint64_t db = tc::desc_k_sw128(sb + Lay::kKps * Lay::kA + u * Lay::kB);
+            const uint64_t da = tc::desc_k_sw128(a0 + t * Lay::kA);
+            const uint64_t db = tc::desc_k_sw128(b0 + (two ? 0 : t * Lay::kB));
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              if (FP8)
-                tc::mma_f8(d, da + 2u * k, db + 2u * k, idesc,
-                           (kt > 0 || k > 0) ? 1u : 0u);
-              else
-                tc::mma_f16(d, da + 2u * k, db + 2u * k, idesc,
-                            (kt > 0 || k > 0) ? 1u : 0u);
+              const uint32_t acc = (u > 0 || t > 0 || k > 0) ? 1u : 0u;
+              if (FP8) tc::mma_f8(d, da + 2u * k, db + 2u * k, idesc, acc);
+              else tc::mma_f16(d, da + 2u * k, db + 2u * k, idesc, acc);
             }
           }
-          tc::mma_commit(&empty[stage]);
-          if (++stage == (uint32_t)STAGES) { stage = 0; phase ^= 1; }
+          tc::mma_commit(&sempty[ss]);
+          if (++ss == (uint32_t)ns) { ss = 0; sphase ^= 1; }
+          if (streamed) {
+            tc::mma_commit(&jempty[js]);
+            if (++js == (uint32_t)nj) { js = 0; jphase ^= 1; }
+          }
         }
         if (ok) tc::mma_commit(&acc_full[g]);
         ISING_RTRACE(2, s, g);
@@ -2152,7 +2165,7 @@ struct TcState {
   bool small = false;     // small form (n <= 128): all of J per CTA, spins kept on chip
   size_t small_bytes = 0;
   int small_grid = 0;     // small form: CTAs (one per block of gn restarts)
-  int jres = 0, nst = 0;  // resident form: J tiles kept in shared memory, stages
+  int ru = 0, nj = 0, ns = 0;  // resident form: resident units, ring slots
   uint32_t bars = 0;      // resident form: offset of the barrier block
   size_t res_bytes = 0;   // resident form: dynamic shared memory
   DevMem err;
@@ -2500,15 +2513,28 @@ int tc_setup(ising_ds* ds) {
       if (!gn && fits(c)) gn = c;
     if (!gn && fits(128)) gn = 64, gr = 2;
     if (gn) {
-      // shared memory: resident J tiles (as many as leave room for 4 stages of
-      // 2 k-blocks), then the stages, then the barrier block
-      const int64_t kA = (int64_t)kBM * kRowBytes, kStage = 2 * (kA + (int64_t)gn * kRowBytes);
+      // shared memory: resident units, the J and the S ring, the barrier block
+      const int64_t kJ = 2 * (int64_t)kBM * kRowBytes;
+      const int64_t kS = (int64_t)gn * kRowBytes * (ds->planes == 2 ? 1 : 2);
       const int64_t region = ((int64_t)ctx->smem_optin - 1024 - 512) / 1024 * 1024;
-      const int nkt = ceil_div_i(ds->n, st->fp8 ? 128 : 64) * ds->planes;
-      const int jres = (int)std::min<int64_t>(nkt, std::max<int64_t>(0, (region - 4 * kStage) / kA));
-      const int nst = (int)std::min<int64_t>(8, (region - jres * kA) / kStage);
+      const int units = (ceil_div_i(ds->n, st->fp8 ? 128 : 64) * ds->planes + 1) / 2;
+      // the split of the room between resident units and the two rings by the
+      // time a phase's copies take: a ring moves its bytes per round trip
+      // (about 2 us from L2 under load), both together at most 90 GB/s per SM
+      int ns = 2, nj = 0, ru = -1;
+      double best = 0.0;
+      for (int cs = 2; cs <= 16; ++cs)
+        for (int cj = 0; cj <= 8; ++cj) {
+          const int64_t left = region - cs * kS - cj * kJ;
+          const int cr = (int)std::min<int64_t>(units, left < 0 ? -1 : left / kJ);
+          if (cr < 0 || (cr < units) != (cj >= 2) || (cr == units && cj > 0)) continue;
+          const double js = (double)(units - cr) * kJ, sb = (double)units * kS;
+          const double t = std::max({cj ? js / (cj * (double)kJ / 2.0) : 0.0, sb / (cs * (double)kS / 2.0),
+                                     (js + sb) / 90e3});
+          if (ru < 0 || t < best - 1e-9) best = t, ns = cs, nj = cj, ru = cr;
+        }
       int nb = 0;
-      if (nst >= 2) {
+      if (ru >= 0) {
         const size_t bytes = (size_t)region + 512 + 1024;
         if (gr == 2) ISING_TRY((resident_attr_bn<64, 2>(ds, st->fp8, bytes, &nb)));
         else if (gn == 64) ISING_TRY((resident_attr_bn<64, 1>(ds, st->fp8, bytes, &nb)));
@@ -2520,8 +2546,9 @@ int tc_setup(ising_ds* ds) {
           st->gr = gr;
           st->res_grid = mt * ceil_div_i(ds->B, gr * gn);
           st->BN = ds->B <= 64 ? 64 : 128;  // (the final evaluation's tiles)
-          st->jres = jres;
-          st->nst = nst;
+          st->ru = ru;
+          st->nj = nj;
+          st->ns = ns;
           st->bars = (uint32_t)region;
           st->res_bytes = bytes;
         }
@@ -2757,14 +2784,15 @@ int tc_run_resident(ising_ds* ds, int64_t steps) {
   r.chs = ds->inst.ch * std::ldexp(1.0, -ds->h_shift);
   r.rows = ds->mtiles;
   r.slice = ceil_div_i(st->gn, ceil_div_i(ds->n, kBM));
-  r.jres = st->jres;
+  r.ru = st->ru;
+  r.nj = st->nj;
+  r.ns = st->ns;
   r.T = ds->T;
   const bool conv = ds->conv.p != nullptr;
   r.conv_ring = conv ? ds->conv_ring() : nullptr;
   r.conv_init = conv ? ds->conv_init() : nullptr;
   r.conv_step = conv ? ds->conv_step() : nullptr;
   r.conv_count = conv ? ds->conv_count() : nullptr;
-  r.nst = st->nst;
   r.bars = st->bars;
   r.nfull = st->nfull;
   if (st->gr == 2) return resident_launch_bn<64, 2>(ds, st, r);
