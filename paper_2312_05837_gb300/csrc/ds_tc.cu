@@ -69,6 +69,7 @@ struct TcArgs {
   int planes;  // 1 or 2
   int f16;     // 16-bit operands are FP16 (else BF16): MMA input format and spin encoding
   int mtiles, ntiles;
+  int balanced = 0;  // pair-MMA streaming kernel: tiles of several widths (balanced_tile)
   StepConsts k;
   const float2* bias;
   const long long* counters;
@@ -212,6 +213,7 @@ struct TileRef {
   long long* hpart;
   float* epart;
   int mt, m0, n0;
+  int width;  // restarts of the tile, a multiple of 32
   bool skip;  // every restart of the tile has stopped (convergence rule)
   __device__ const CUtensorMap* a(int plane) const { return plane == 0 ? A0 : (plane == 1 ? A1 : A2); }
   __device__ const CUtensorMap* j2(int plane) const { return plane == 0 ? J0 : (plane == 1 ? J1 : J2); }
@@ -236,6 +238,50 @@ __device__ __forceinline__ void advance_counters(unsigned long long* done, long 
   __threadfence();
 }
 
+// Operand maps of one spin slot per tile width: boxes of 32 (k + 1) restarts
+// (half of that for CTA pairs).
+struct WidthMaps {
+  CUtensorMap m[8];
+};
+
+// Tiles of the pair-MMA form that share a step's work out evenly: the columns
+// of all row tiles in order, in units of 32 restarts, are dealt in waves. Every
+// pair takes the same width in a wave, the widest first, so that its units add
+// up to ceil(units / pairs) and its last tile, whose epilogue no MMAs hide, is
+// the narrowest. A range that crosses into the next row tile makes two tiles.
+// Within a wave neighbours share row tiles, as with tiles of one width. At 4096
+// spins x 4096 restarts, 76 pairs take 27 units as 8 + 8 + 8 + 3: 167 us per step
+// against 171 for four tiles of 7. (The other forms keep one width: with a
+// width known only at run time their epilogue spills.) A tile is coded as 16
+// first unit + units.
+__device__ __forceinline__ int wave_width(int wave, int per_group, int widest) {
+  const int full = per_group / widest, rest = per_group - full * widest;
+  if (rest == 1 && full > 0) {
+    // (a single unit costs nearly the MMA time of two)
+    return wave < full - 1 ? widest : (wave == full - 1 ? widest - 1 : (wave == full ? 2 : 0));
+  }
+  return wave < full ? widest : (wave == full ? rest : 0);
+}
+
+// The j-th tile of `group`, or 16 total. (Not inlined: its values would stay in
+// registers through the tile loops, whose epilogue has none to spare.)
+__device__ __noinline__ int balanced_tile(int total, int per_row, int groups, int group, int widest,
+                                          int j) {
+  const int per_group = (total + groups - 1) / groups;
+  int base = 0;
+  for (int wave = 0, w; (w = wave_width(wave, per_group, widest)) > 0; ++wave) {
+    int a = base + group * w;
+    const int b = min(a + w, total);
+    while (a < b) {
+      const int len = min(b - a, per_row - a % per_row);
+      if (j-- == 0) return a * 16 + len;
+      a += len;
+    }
+    base += groups * w;
+  }
+  return total * 16;
+}
+
 // Tiles of one instance: everything comes from the kernel's parameters (the
 // host chose the slots of step t), tiles numbered row tile by row tile.
 template <int BN>
@@ -245,7 +291,7 @@ struct OneInstance {
   static constexpr bool kSplit = false;
   static constexpr bool kFold = true;  // may track the previous step (TcArgs::fold)
   const TcArgs& P;  // the kernel's parameter
-  const CUtensorMap *A0, *A1, *A2, *B, *J0, *J1, *J2, *S2;
+  const CUtensorMap *A0, *A1, *A2, *J0, *J1, *J2, *B, *S2;
   __device__ int first() const { return blockIdx.x; }
   __device__ int stride() const { return gridDim.x; }
   // the CTA's j-th tile
@@ -273,16 +319,17 @@ struct OneInstance {
     r.P = &P;
     r.A0 = A0; r.A1 = A1; r.A2 = A2;
     r.J0 = J0; r.J1 = J1; r.J2 = J2;
-    r.B = B;
-    r.S2 = S2;
     r.S = P.S;
     r.Snext = P.Snext;
     r.qpart = P.qpart;
     r.hpart = P.hpart;
     r.epart = P.epart;
+    r.B = B;
+    r.S2 = S2;
     r.mt = tl / P.ntiles;
     r.m0 = r.mt * kBM;
     r.n0 = (tl % P.ntiles) * BN;
+    r.width = BN;
     r.skip = restarts_retired(P.live32, r.n0, min((int64_t)r.n0 + BN, P.B));
     return r;
   }
@@ -378,6 +425,7 @@ struct PackedInstances {
     r.mt = local / e.args.ntiles;
     r.m0 = r.mt * kBM;
     r.n0 = (local % e.args.ntiles) * BN;
+    r.width = BN;
     r.skip = restarts_retired(e.args.live32, r.n0, min((int64_t)r.n0 + BN, e.args.B));
     return r;
   }
@@ -402,14 +450,22 @@ struct PairInstance {
   static constexpr bool kSplit = SPLIT;
   static constexpr bool kFold = true;
   const TcArgs& P;
-  const CUtensorMap *A0, *A1, *A2, *B, *J0, *J1, *J2, *S2;
-  const CUtensorMap* Bh;  // S_t, boxes of one k-block x BN / 2 restarts
+  const CUtensorMap *A0, *A1, *A2, *J0, *J1, *J2;
+  const WidthMaps* Bh;  // S_t, boxes of one k-block x half of a tile's restarts
   uint32_t rank;
   __device__ int first() const { return (int)tc::cluster_index(); }
   __device__ int stride() const { return (int)tc::cluster_count(); }
   // the CTA's j-th tile (row-tile-major order)
-  __device__ int at(int j) const { return first() + j * stride(); }
-  __device__ int total() const { return (P.mtiles + 1) / 2 * P.ntiles; }
+  __device__ int at(int j) const {
+    const int per_row = (int)((P.B + 31) / 32);
+    if (SPLIT && P.balanced)
+      return balanced_tile((P.mtiles + 1) / 2 * per_row, per_row, stride(), first(), BN / 32, j);
+    return first() + j * stride();
+  }
+  __device__ int total() const {
+    return SPLIT && P.balanced ? (P.mtiles + 1) / 2 * (int)((P.B + 31) / 32) * 16
+                               : (P.mtiles + 1) / 2 * P.ntiles;
+  }
   __device__ int* err() const { return P.err; }
   __device__ unsigned long long* trace() const { return P.trace; }
   __device__ bool fused() const { return P.planes == 2; }
@@ -430,17 +486,25 @@ struct PairInstance {
     r.P = &P;
     r.A0 = A0; r.A1 = A1; r.A2 = A2;
     r.J0 = J0; r.J1 = J1; r.J2 = J2;
-    r.B = Bh;
-    r.S2 = S2;
     r.S = P.S;
     r.Snext = P.Snext;
     r.qpart = P.qpart;
     r.hpart = P.hpart;
     r.epart = P.epart;
-    r.mt = 2 * (tl / P.ntiles) + (int)rank;
+    if (SPLIT && P.balanced) {
+      const int per_row = (int)((P.B + 31) / 32);
+      r.mt = 2 * ((tl >> 4) / per_row) + (int)rank;
+      r.n0 = (tl >> 4) % per_row * 32;
+      r.width = (tl & 15) * 32;
+      r.skip = false;
+    } else {
+      r.mt = 2 * (tl / P.ntiles) + (int)rank;
+      r.n0 = (tl % P.ntiles) * BN;
+      r.width = BN;
+      r.skip = restarts_retired(P.live32, r.n0, min((int64_t)r.n0 + BN, P.B));
+    }
     r.m0 = r.mt * kBM;
-    r.n0 = (tl % P.ntiles) * BN;
-    r.skip = restarts_retired(P.live32, r.n0, min((int64_t)r.n0 + BN, P.B));
+    r.B = r.S2 = &Bh->m[r.width / 32 - 1];
     return r;
   }
 };
@@ -529,6 +593,9 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
         // k-steps of the ring: k-blocks (fused), else k-blocks of each plane
         const int nkt = fused ? nk : nk * planes;
         const int kps = fused ? 1 : Lay::kKps;
+        // S rows of this tile in this CTA's stage
+        const int srows = SPLIT ? T.width / 2 : T.width;
+        const uint32_t sbytes = (uint32_t)srows * kRowBytes;
         if (Src::kGlobalMaps) {
           if (jside) {
             for (int p = 0; p < planes; ++p) {
@@ -552,7 +619,7 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
           // barrier, whose producers expect both CTAs' bytes
           if (!SPLIT || lead)
             tc::mbar_expect_tx(&full[stage], (uint32_t)(fused && jside ? planes : cnt) *
-                                                 (jside ? Lay::kA : Lay::kB) * (SPLIT ? 2u : 1u));
+                                                 (jside ? Lay::kA : sbytes) * (SPLIT ? 2u : 1u));
           const uint32_t lead_full = SPLIT ? tc::mapa(tc::smem_u32(&full[stage]), 0) : 0u;
           const int plane0 = kt0 / nk, kb0 = kt0 - plane0 * nk;
           if (fused) {
@@ -568,10 +635,10 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
               }
             } else if constexpr (SPLIT) {
               if (lead) tc::tma_load_2d_hint(sb, T.B, &full[stage], kb * kBK, T.n0, pol);
-              else tc::tma_load_2d_to_pair(sb, T.B, lead_full, kb * kBK, T.n0 + BN / 2, pol);
+              else tc::tma_load_2d_to_pair(sb, T.B, lead_full, kb * kBK, T.n0 + srows, pol);
             } else if constexpr (Src::kPair) {
-              tc::tma_load_2d_mc(sb + src.rank * (BN / 2) * kRowBytes, T.B, &full[stage], kb * kBK,
-                                 T.n0 + (int)src.rank * (BN / 2), 0x3, pol);
+              tc::tma_load_2d_mc(sb + src.rank * (srows / 2) * kRowBytes, T.B, &full[stage], kb * kBK,
+                                 T.n0 + (int)src.rank * (srows / 2), 0x3, pol);
             } else {
               tc::tma_load_2d_hint(sb, T.B, &full[stage], kb * kBK, T.n0, pol);
             }
@@ -597,16 +664,16 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
                     tc::tma_load_2d_to_pair(sa, T.a(plane), lead_full, kb * kBK, T.m0, pol);
                   else
                     tc::tma_load_2d_to_pair(sa + Lay::kA, T.B, lead_full, kb * kBK,
-                                            T.n0 + BN / 2, pol);
+                                            T.n0 + srows, pol);
                 }
               } else if (jside) {
                 tc::tma_load_2d_hint(sa + u * Lay::kA, T.a(plane), &full[stage], kb * kBK, T.m0, pol);
               } else if constexpr (Src::kPair) {
                 // this CTA's half of the spin tile, to both CTAs of the pair
-                tc::tma_load_2d_mc(sa + Lay::kA + src.rank * (BN / 2) * kRowBytes, T.B,
-                                   &full[stage], kb * kBK, T.n0 + (int)src.rank * (BN / 2), 0x3, pol);
+                tc::tma_load_2d_mc(sa + Lay::kA + src.rank * (srows / 2) * kRowBytes, T.B,
+                                   &full[stage], kb * kBK, T.n0 + (int)src.rank * (srows / 2), 0x3, pol);
               } else {
-                tc::tma_load_2d_hint(sa + Lay::kKps * Lay::kA + u * Lay::kB, T.B, &full[stage],
+                tc::tma_load_2d_hint(sa + Lay::kKps * Lay::kA + u * sbytes, T.B, &full[stage],
                                      kb * kBK, T.n0, pol);
               }
             }
@@ -653,7 +720,8 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
         const int planes = P.planes;
         const int nkt = fused ? P.nk : P.nk * planes;
         const int kps = fused ? 1 : Lay::kKps;
-        const uint32_t idesc = op_idesc(BN, FP8, P.f16, SPLIT ? 256 : 128);
+        const uint32_t idesc = op_idesc(T.width, FP8, P.f16, SPLIT ? 256 : 128);
+        const uint32_t sbytes = (uint32_t)(SPLIT ? T.width / 2 : T.width) * kRowBytes;
         const int buf = it & 1;
         const uint32_t use = (uint32_t)(it >> 1);
         // (split pairs: both CTAs' epilogues release it, from the cluster)
@@ -693,7 +761,7 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
             if (kt >= nkt) break;
             // descriptors of the tiles; K step k adds 32 bytes (2 in the >> 4 address field)
             const uint64_t da = tc::desc_k_sw128(sb + u * Lay::kA);
-            const uint64_t db = tc::desc_k_sw128(sb + Lay::kKps * Lay::kA + u * Lay::kB);
+            const uint64_t db = tc::desc_k_sw128(sb + Lay::kKps * Lay::kA + u * sbytes);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {  // 32 bytes of K per MMA (16 BF16 or 32 E4M3)
               const uint32_t acc = (kt > 0 || k > 0) ? 1u : 0u;
@@ -732,7 +800,6 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
     // ------------------------------------------------ epilogue
     const int q = warp & 3;             // TMEM lane quarter of this warp
     const int part = (warp - 4) >> 2;   // which quarter of the tile's columns
-    constexpr int kCols = BN / 4;
     if constexpr (MODE == kModeUpdate && Src::kFold) {
       // the previous step's best tracking, a warp per restart over all the
       // launch's epilogue warps, while the MMAs of the first tile run (it
@@ -760,10 +827,11 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
       const uint32_t use = (uint32_t)(my_it >> 1);
       const int mt = T.mt;
       const int64_t m0 = T.m0;
-      const int64_t n0 = (int64_t)T.n0 + part * kCols;
+      const int cols = T.width / 4;  // of this warp's part
+      const int64_t n0 = (int64_t)T.n0 + part * cols;
       if ((MODE == kModeUpdate || MODE == kModeRelaxed) && P.work && mt == 0 && warp == 4 &&
           lane == 0)
-        atomicAdd(P.work, (unsigned long long)min((int64_t)BN, P.B - T.n0));
+        atomicAdd(P.work, (unsigned long long)min((int64_t)T.width, P.B - T.n0));
       if (!tc::mbar_wait(&acc_full[buf], use & 1, abort_flag, kWaitCycles)) {
         atomicExch(src.err(), 3);
         break;
@@ -776,9 +844,9 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
       const int hi = row_ok ? P.hint[i] : 0;
       const float rs = (P.rowscale && row_ok) ? P.rowscale[i] : 1.f;
       const uint32_t tbase = tmem_base + ((uint32_t)(32 * q) << 16) +
-                             (uint32_t)(buf * BN + part * kCols);
+                             (uint32_t)(buf * BN + part * cols);
 #pragma unroll 1
-      for (int c0 = 0; c0 < kCols; c0 += kChunk) {
+      for (int c0 = 0; c0 < cols; c0 += kChunk) {
         uint32_t r[kChunk];
         tc::tmem_ld8(tbase + c0, r);
         // state of this chunk's restarts, loaded while the TMEM read lands
@@ -808,7 +876,7 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
           }
         }
         tc::tmem_wait_ld();
-        if (c0 + kChunk == kCols) {
+        if (c0 + kChunk == cols) {
           tc::fence_before_sync();
           __syncwarp();
           if (lane == 0) {
@@ -908,7 +976,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                    const __grid_constant__ CUtensorMap tmJ2_1,
                    const __grid_constant__ CUtensorMap tmJ2_2,
                    const __grid_constant__ CUtensorMap tmS2, const __grid_constant__ TcArgs P) {
-  const OneInstance<BN> src{P, &tmA0, &tmA1, &tmA2, &tmB, &tmJ2_0, &tmJ2_1, &tmJ2_2, &tmS2};
+  const OneInstance<BN> src{P, &tmA0, &tmA1, &tmA2, &tmJ2_0, &tmJ2_1, &tmJ2_2, &tmB, &tmS2};
   step_tiles<BN, MODE, INT_E, FP8>(src);
 }
 
@@ -918,13 +986,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     tc_step_pair_kernel(const __grid_constant__ CUtensorMap tmA0,
                         const __grid_constant__ CUtensorMap tmA1,
                         const __grid_constant__ CUtensorMap tmA2,
-                        const __grid_constant__ CUtensorMap tmBh,
+                        const __grid_constant__ WidthMaps tmBh,
                         const __grid_constant__ CUtensorMap tmJ2_0,
                         const __grid_constant__ CUtensorMap tmJ2_1,
                         const __grid_constant__ CUtensorMap tmJ2_2,
-                        const __grid_constant__ CUtensorMap tmS2, const __grid_constant__ TcArgs P) {
-  const PairInstance<BN> src{P,      &tmA0,   &tmA1,   &tmA2, &tmBh, &tmJ2_0,
-                             &tmJ2_1, &tmJ2_2, &tmS2,   &tmBh, tc::cluster_rank()};
+                        const __grid_constant__ TcArgs P) {
+  const PairInstance<BN> src{P,       &tmA0,   &tmA1, &tmA2, &tmJ2_0,
+                             &tmJ2_1, &tmJ2_2, &tmBh, tc::cluster_rank()};
   step_tiles<BN, MODE, INT_E, FP8>(src);
 }
 
@@ -934,13 +1002,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     tc_step_split_kernel(const __grid_constant__ CUtensorMap tmA0,
                          const __grid_constant__ CUtensorMap tmA1,
                          const __grid_constant__ CUtensorMap tmA2,
-                         const __grid_constant__ CUtensorMap tmBh,
+                         const __grid_constant__ WidthMaps tmBh,
                          const __grid_constant__ CUtensorMap tmJ2_0,
                          const __grid_constant__ CUtensorMap tmJ2_1,
                          const __grid_constant__ CUtensorMap tmJ2_2,
-                         const __grid_constant__ CUtensorMap tmS2, const __grid_constant__ TcArgs P) {
-  const PairInstance<BN, true> src{P,      &tmA0,   &tmA1, &tmA2, &tmBh, &tmJ2_0,
-                                   &tmJ2_1, &tmJ2_2, &tmS2, &tmBh, tc::cluster_rank()};
+                         const __grid_constant__ TcArgs P) {
+  const PairInstance<BN, true> src{P,       &tmA0,   &tmA1, &tmA2, &tmJ2_0,
+                                   &tmJ2_1, &tmJ2_2, &tmBh, tc::cluster_rank()};
   step_tiles<BN, MODE, INT_E, FP8>(src);
 }
 
@@ -2144,8 +2212,8 @@ struct TcState {
   // resident kernel: views of J (per plane) and of the spin slots as
   // [k-block][row][128 B] with boxes of two whole k-blocks
   CUtensorMap J2[3], S2[3];
-  CUtensorMap SP[3];  // streaming kernel: the spin slots' pair views, boxes of BN restarts
-  CUtensorMap Bh[3];  // pair tiles: the spin slots, boxes of BN / 2 restarts
+  CUtensorMap SP[3];  // streaming kernel: the spin slots' views of two k-blocks, boxes of BN restarts
+  WidthMaps Bh[3];    // pair tiles: the spin slots, boxes of half the widths
   bool pair = false;  // streaming kernel over clusters of two CTAs sharing spin tiles
   bool split = false; // ... whose MMAs run as one per pair (cta_group::2)
   int nfull = 0;      // k-blocks lying wholly below column n (0 in the small form)
@@ -2226,7 +2294,7 @@ int make_map_pairs(ising_ctx* ctx, CUtensorMap* map, const void* base, int64_t n
 
 template <int BN, int MODE, bool INT_E, bool FP8>
 int launch_bn(ising_ds* ds, TcState* st, const TcArgs& a, const CUtensorMap& mB,
-              const CUtensorMap& mS2, const CUtensorMap& mBh) {
+              const CUtensorMap& mS2, const WidthMaps& mBh) {
   const size_t smem = TcLayout<BN>::kBytes;
   if constexpr (BN >= 192) {
     if (st->pair && st->split) {
@@ -2238,11 +2306,11 @@ int launch_bn(ising_ds* ds, TcState* st, const TcArgs& a, const CUtensorMap& mB,
                                                  (int)ssmem));
         attr_set = true;
       }
-      const int pairs = (a.mtiles + 1) / 2 * a.ntiles;
+      const int pairs = (a.mtiles + 1) / 2 * (a.balanced ? ceil_div_i(a.B, 32) : a.ntiles);
       const int clusters = std::max(1, std::min(pairs, ds->ctx->sm_count / 2));
       kern<<<2 * clusters, kThreads, ssmem, ds->ctx->stream>>>(st->A[0], st->A[1], st->A[2], mBh,
                                                                st->J2[0], st->J2[1], st->J2[2],
-                                                               mS2, a);
+                                                               a);
       ISING_CUDA(ds->ctx, cudaGetLastError());
       return ISING_OK;
     }
@@ -2259,7 +2327,7 @@ int launch_bn(ising_ds* ds, TcState* st, const TcArgs& a, const CUtensorMap& mB,
       const int clusters = std::max(1, std::min(pairs, ds->ctx->sm_count / 2));
       kern<<<2 * clusters, kThreads, smem, ds->ctx->stream>>>(st->A[0], st->A[1], st->A[2], mBh,
                                                               st->J2[0], st->J2[1], st->J2[2],
-                                                              mS2, a);
+                                                              a);
       ISING_CUDA(ds->ctx, cudaGetLastError());
       return ISING_OK;
     }
@@ -2279,7 +2347,7 @@ int launch_bn(ising_ds* ds, TcState* st, const TcArgs& a, const CUtensorMap& mB,
 
 template <int MODE, bool INT_E, bool FP8>
 int launch_bn_sel(ising_ds* ds, TcState* st, const TcArgs& a, const CUtensorMap& mB,
-                  const CUtensorMap& mS2, const CUtensorMap& mBh) {
+                  const CUtensorMap& mS2, const WidthMaps& mBh) {
   switch (st->BN) {
     case 256: return launch_bn<256, MODE, INT_E, FP8>(ds, st, a, mB, mS2, mBh);
     case 224: return launch_bn<224, MODE, INT_E, FP8>(ds, st, a, mB, mS2, mBh);
@@ -2290,7 +2358,7 @@ int launch_bn_sel(ising_ds* ds, TcState* st, const TcArgs& a, const CUtensorMap&
 
 template <int MODE, bool INT_E>
 int launch_mode(ising_ds* ds, TcState* st, const TcArgs& a, const CUtensorMap& mB,
-                const CUtensorMap& mS2, const CUtensorMap& mBh) {
+                const CUtensorMap& mS2, const WidthMaps& mBh) {
   return st->fp8 ? launch_bn_sel<MODE, INT_E, true>(ds, st, a, mB, mS2, mBh)
                  : launch_bn_sel<MODE, INT_E, false>(ds, st, a, mB, mS2, mBh);
 }
@@ -2301,7 +2369,7 @@ template <bool INT_E>
 int launch_relaxed(ising_ds* ds, TcState* st, const TcArgs& a, const CUtensorMap& mB,
                    const CUtensorMap& mS2) {
   if (st->fp8) return fail(ds->ctx, ISING_ENOTSUP, "relaxed product needs BF16 operands");
-  return launch_bn_sel<kModeRelaxed, INT_E, false>(ds, st, a, mB, mS2, mB);
+  return launch_bn_sel<kModeRelaxed, INT_E, false>(ds, st, a, mB, mS2, st->Bh[0]);
 }
 
 }  // namespace
@@ -2566,22 +2634,20 @@ int tc_setup(ising_ds* ds) {
 // common allocation; they are built on first use.
 static int tc_maps(ising_ds* ds, TcState* st) {
   static_assert(sizeof(CUtensorMap) == 128, "CUtensorMap size");
+  const int kb = st->fp8 ? 128 : 64;
   for (int s = 0; s < 3; ++s) {
-    ISING_TRY(make_map(ds->ctx, &st->B[s], ds->spins[s].p, ds->n, ds->B, ds->ld,
-                       st->fp8 ? 128 : 64, st->BN, st->fp8));
-    if (st->nfull >= 2) {
-      ISING_TRY(make_map_pairs(ds->ctx, &st->SP[s], ds->spins[s].p, st->nfull, ds->B, ds->ld, st->BN,
-                               st->fp8));
-      if (st->resident)
-        ISING_TRY(make_map_pairs(ds->ctx, &st->S2[s], ds->spins[s].p, st->nfull, ds->B, ds->ld,
-                                 st->gn, st->fp8));
-    }
-    if (st->resident)
-      ISING_TRY(make_map(ds->ctx, &st->Bg[s], ds->spins[s].p, ds->n, ds->B, ds->ld,
-                         st->fp8 ? 128 : 64, st->gn, st->fp8));
+    const void* sp = ds->spins[s].p;
+    ISING_TRY(make_map(ds->ctx, &st->B[s], sp, ds->n, ds->B, ds->ld, kb, st->BN, st->fp8));
+    if (st->nfull >= 2)
+      ISING_TRY(make_map_pairs(ds->ctx, &st->SP[s], sp, st->nfull, ds->B, ds->ld, st->BN, st->fp8));
     if (st->pair)
-      ISING_TRY(make_map(ds->ctx, &st->Bh[s], ds->spins[s].p, ds->n, ds->B, ds->ld,
-                         st->fp8 ? 128 : 64, st->BN / 2, st->fp8));
+      for (int w = 32; w <= st->BN; w += 32)
+        ISING_TRY(make_map(ds->ctx, &st->Bh[s].m[w / 32 - 1], sp, ds->n, ds->B, ds->ld, kb, w / 2, st->fp8));
+    if (st->resident) {
+      ISING_TRY(make_map(ds->ctx, &st->Bg[s], sp, ds->n, ds->B, ds->ld, kb, st->gn, st->fp8));
+      if (st->nfull >= 2)
+        ISING_TRY(make_map_pairs(ds->ctx, &st->S2[s], sp, st->nfull, ds->B, ds->ld, st->gn, st->fp8));
+    }
   }
   if (st->nfull >= 2)
     for (int p = 0; p < 3; ++p)
@@ -2610,6 +2676,8 @@ int tc_run(ising_ds* ds, int mode, float* Gout) {
   a.f16 = st->f16 ? 1 : 0;
   a.mtiles = ceil_div_i(ds->n, kBM);
   a.ntiles = ceil_div_i(ds->B, st->BN);
+  // (tiles retire as a whole under the convergence rule: one width then)
+  a.balanced = ds->live.p == nullptr;
   a.k = ds->k;
   a.bias = ds->bias.as<float2>();
   a.counters = ds->counters.as<long long>();
@@ -2638,12 +2706,12 @@ int tc_run(ising_ds* ds, int mode, float* Gout) {
     a.trk = track_args(ds);
   }
   if (ds->p.flags & ISING_DS_PROFILE) {
-    if (!st->trace.p) ISING_TRY(dev_alloc(ds->ctx, st->trace, (size_t)std::max(st->grid, st->res_grid) * 8 * 8));
+    if (!st->trace.p) ISING_TRY(dev_alloc(ds->ctx, st->trace, (size_t)std::max({st->grid, st->res_grid, ds->ctx->sm_count}) * 8 * 8));
     a.trace = st->trace.as<unsigned long long>();
   }
   const CUtensorMap& mS = st->B[t % 3];
   const CUtensorMap& mS2 = st->SP[t % 3];
-  const CUtensorMap& mSh = st->Bh[t % 3];
+  const WidthMaps& mSh = st->Bh[t % 3];
   a.nfull = st->nfull;
   const bool ie = ds->int_energy;
   switch (mode) {
@@ -2656,6 +2724,7 @@ int tc_run(ising_ds* ds, int mode, float* Gout) {
       // x_{t+1} (x has no pair view: one copy per k-block)
       const CUtensorMap& mX = st->Bx[t % 2];
       a.nfull = 0;
+      a.balanced = 0;
       return ie ? launch_relaxed<true>(ds, st, a, mX, mS2) : launch_relaxed<false>(ds, st, a, mX, mS2);
     }
     default: return launch_mode<kModeCoupling, true>(ds, st, a, mS, mS2, mSh);
@@ -2763,7 +2832,7 @@ int tc_run_resident(ising_ds* ds, int64_t steps) {
   a.live32 = nullptr;  // the resident forms do not retire restarts
   a.work = nullptr;
   if (ds->p.flags & ISING_DS_PROFILE) {
-    if (!st->trace.p) ISING_TRY(dev_alloc(ds->ctx, st->trace, (size_t)std::max(st->grid, st->res_grid) * 8 * 8));
+    if (!st->trace.p) ISING_TRY(dev_alloc(ds->ctx, st->trace, (size_t)std::max({st->grid, st->res_grid, ds->ctx->sm_count}) * 8 * 8));
     a.trace = st->trace.as<unsigned long long>();
   }
   r.steps = steps;
