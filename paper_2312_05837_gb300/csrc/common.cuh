@@ -226,6 +226,10 @@ __device__ __forceinline__ int32_t load_as_int(const void* p, int dt, int64_t i)
 int energy_device(ising_ctx* ctx, const DevInstance& inst, const int8_t* spins,
                   int64_t count, double* E, int64_t* Q, int64_t* H);
 
+// Energies of integer-valued FP16 planes on the tensor cores; defined in ds_tc.cu.
+int tc_plane_energies(ising_ctx* ctx, int64_t n, int64_t ld, int64_t count, const uint16_t* planes,
+                      int nplanes, const void* S, long long* parts);
+
 // SplitMix64 output number `counter` from `seed` (Steele, Lea, Flood 2014).
 __host__ __device__ __forceinline__ uint64_t splitmix64(uint64_t seed, uint64_t counter) {
   uint64_t z = seed + (counter + 1ull) * 0x9E3779B97F4A7C15ull;

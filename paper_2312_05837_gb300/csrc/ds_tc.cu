@@ -3043,6 +3043,68 @@ int tc_pack_launch(ising_ctx* ctx, uint64_t key, int bn, const void* entries, co
   }
 }
 
+// s^T (plane s) of `count` FP16 +-1 vectors S [count][ld] for each of `planes`
+// integer-valued FP16 planes [planes][n][ld] (n max |plane value| <= 2^22, so
+// the FP32 sums are exact): the streaming kernel's energy mode, a launch per
+// plane. parts [planes][4 ceil(n / 128)][count] receives the partial sums.
+int tc_plane_energies(ising_ctx* ctx, int64_t n, int64_t ld, int64_t count, const uint16_t* planes,
+                      int nplanes, const void* S, long long* parts) {
+  if (ctx->smem_optin < TcLayout<256>::kBytes)
+    return fail(ctx, ISING_ENOTSUP, "device lacks the shared memory the tensor-core step needs");
+  ising_ds ds;
+  ds.ctx = ctx;
+  TcState st;
+  st.f16 = true;
+  st.nfull = (int)(n / 64);
+  const int mt = ceil_div_i(n, kBM);
+  // the narrowest tiles that give every one its own SM
+  st.BN = 256;
+  for (int w : {128, 64})
+    if ((int64_t)mt * ceil_div_i(count, w) <= ctx->sm_count) st.BN = w;
+  const int nt = ceil_div_i(count, st.BN);
+  st.grid = std::max(1, (int)std::min<int64_t>((int64_t)mt * nt, ctx->sm_count));
+  ISING_TRY(make_map(ctx, &st.B[0], S, n, count, ld, 64, st.BN, false));
+  if (st.nfull >= 2) ISING_TRY(make_map_pairs(ctx, &st.SP[0], S, st.nfull, count, ld, st.BN, false));
+  // zeros: step counter, bias table, field, field energies, error word
+  DevMem zero, hpart;
+  const int64_t rows = 4 * (int64_t)mt;
+  ISING_TRY(dev_alloc(ctx, zero, 64 + n * 4));
+  ISING_TRY(dev_alloc(ctx, hpart, (size_t)rows * count * 8));
+  ISING_CUDA(ctx, cudaMemsetAsync(zero.p, 0, 64 + n * 4, ctx->stream));
+  uint8_t* z = zero.as<uint8_t>();
+  for (int p = 0; p < nplanes; ++p) {
+    const uint16_t* plane = planes + (int64_t)p * n * ld;
+    for (int k = 0; k < 3; ++k) {
+      ISING_TRY(make_map(ctx, &st.A[k], plane, n, n, ld, 64, kBM, false));
+      if (st.nfull >= 2) ISING_TRY(make_map_pairs(ctx, &st.J2[k], plane, st.nfull, n, ld, kBM, false));
+    }
+    TcArgs a{};
+    a.n = n;
+    a.B = count;
+    a.ld = ld;
+    a.nk = ceil_div_i(n, 64);
+    a.planes = 1;
+    a.f16 = 1;
+    a.mtiles = mt;
+    a.ntiles = nt;
+    a.counters = reinterpret_cast<const long long*>(z);
+    a.bias = reinterpret_cast<const float2*>(z + 32);
+    a.err = reinterpret_cast<int*>(z + 56);
+    a.hf = reinterpret_cast<const float*>(z + 64);
+    a.hint = reinterpret_cast<const int32_t*>(z + 64);
+    a.S = S;
+    a.qpart = parts + (int64_t)p * rows * count;
+    a.hpart = hpart.as<long long>();
+    a.nfull = st.nfull;
+    ISING_TRY((launch_bn_sel<kModeEnergy, true, false>(&ds, &st, a, st.B[0], st.SP[0], st.Bh[0])));
+  }
+  int e = 0;
+  ISING_CUDA(ctx, cudaMemcpyAsync(&e, z + 56, 4, cudaMemcpyDeviceToHost, ctx->stream));
+  ISING_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  if (e) return fail(ctx, ISING_ETIMEOUT, "tensor-core energies: a bounded wait gave up (role %d)", e);
+  return ISING_OK;
+}
+
 void tc_release(ising_ds* ds) {
   delete static_cast<TcState*>(ds->tc);
   ds->tc = nullptr;

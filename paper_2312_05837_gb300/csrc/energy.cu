@@ -1,9 +1,11 @@
 // K3: energy of rounded spin vectors, E(s) = cQ s^T J s + cH h^T s (Sec. II).
 //
-// Three forms, all deterministic; integer couplings are exact in each:
+// Four forms, all deterministic; integer couplings are exact in each:
 //   fixed    dense J: every J_ij becomes a 64-bit integer (itself, or
 //            rint(J_ij 2^k) with one scale for the matrix), so s^T J s is summed
 //            in integers whatever the order, rounded once at the end;
+//   planes   dense J and many vectors: the same integers as digits in FP16
+//            planes, their sums on the tensor cores, exact as well;
 //   packed   CSR, 8 or more vectors: a lane per vector, spins as bits;
 //   general  a warp per row and vector, int64 or FP64: few CSR vectors, dense J
 //            whose values spread too widely for one scale, the call without
@@ -313,19 +315,21 @@ __global__ void __launch_bounds__(256) energy_fixed_finish(
 // log2(n^2) 2^-53 sum |J_ij|, 16 at n = 256; a smaller sum has more bits to
 // spare), or else the form is not used. sum |J_ij| is at least the count of
 // non-zeros times their geometric mean, which the mean exponent bounds below.
-bool fixed_scale(const DevInstance& I, bool exact, int* shift) {
-  *shift = 0;
-  if (exact) return true;
-  if (I.j_nonzeros == 0) return true;
-  const int64_t lane_terms = 4 * ((I.n + 1023) / 1024) + 4;
-  int lg = 0;
-  while (((int64_t)1 << lg) < lane_terms) ++lg;
-  const int b = std::min(58, 61 - lg);
+bool scale_for(const DevInstance& I, int b, int* shift) {
   int ex = 0;
   std::frexp(I.j_absmax, &ex);  // |J| < 2^ex
   if ((double)I.j_expsum < (double)(ex - b + 48) * (double)I.j_nonzeros) return false;
   *shift = b - ex;
   return *shift >= -120 && *shift <= 120;  // a float power of two; no result underflows
+}
+
+bool fixed_scale(const DevInstance& I, bool exact, int* shift) {
+  *shift = 0;
+  if (exact || I.j_nonzeros == 0) return true;
+  const int64_t lane_terms = 4 * ((I.n + 1023) / 1024) + 4;
+  int lg = 0;
+  while (((int64_t)1 << lg) < lane_terms) ++lg;
+  return scale_for(I, std::min(58, 61 - lg), shift);
 }
 
 template <typename T, int VEC>
@@ -351,6 +355,100 @@ int fixed_launch_t(ising_ctx* ctx, const DevInstance& I, int shift, const uint32
   // rows of a multiple of four values start on a vector boundary
   return I.n % 4 == 0 ? fixed_launch<T, 4>(ctx, I, shift, bits, words, count, limbs)
                       : fixed_launch<T, 1>(ctx, I, shift, bits, words, count, limbs);
+}
+
+// --------------------------------------------------------------- planes form
+//
+// The integers of the fixed form as digits d_p in [-2^(w - 1), 2^(w - 1)] of base
+// 2^w, one FP16 plane per digit: s^T d_p s is a matrix product whose FP32 sums
+// are exact while n 2^(w - 1) <= 2^22, so 256 vectors cost the tensor cores 5
+// products where the fixed form spends 7 integer instructions per coupling and
+// vector. Bound by writing and reading the planes (10 bytes per coupling).
+
+// Digits of every coupling, and the spins as FP16 +-1.
+template <typename T>
+__global__ void __launch_bounds__(256) split_digits_kernel(const T* __restrict__ J, int64_t n, int64_t ld,
+                                                           int shift, double dscale, int w, int planes,
+                                                           uint16_t* __restrict__ out) {
+  const long long half = 1ll << (w - 1), mask = (1ll << w) - 1;
+  // four columns per thread: one 8-byte store per plane (rows of ld, a multiple
+  // of 64, start on a vector boundary; columns from n to ld are never read)
+  for (int64_t i = blockIdx.y; i < n; i += gridDim.y)
+    for (int64_t k = 4 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x); k < n;
+         k += 4 * (int64_t)gridDim.x * blockDim.x) {
+      long long I[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) I[c] = k + c < n ? to_fixed<T>(J[i * n + k + c], shift, dscale) : 0;
+      for (int p = 0; p < planes; ++p) {
+        uint16_t f[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          // (the last digit takes what is left, at most 2^(w - 1) in magnitude)
+          const long long d = p + 1 < planes ? ((I[c] + half) & mask) - half : I[c];
+          f[c] = __half_as_ushort(__int2half_rn((int)d));
+          I[c] = (I[c] - d) >> w;
+        }
+        *reinterpret_cast<uint2*>(out + ((int64_t)p * n + i) * ld + k) =
+            make_uint2(f[0] | (uint32_t)f[1] << 16, f[2] | (uint32_t)f[3] << 16);
+      }
+    }
+}
+
+__global__ void __launch_bounds__(256) spins_f16_kernel(const int8_t* __restrict__ spins, int64_t count,
+                                                        int64_t n, int64_t ld, uint16_t* __restrict__ out) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count * ld;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t v = e / ld, i = e - v * ld;
+    out[e] = i >= n ? 0 : (spins[v * n + i] == 1 ? 0x3C00 : 0xBC00);
+  }
+}
+
+// sum_p 2^(w p) (sum of plane p's partial rows) in limbs; a warp per vector.
+__global__ void __launch_bounds__(256) join_digits_kernel(int64_t count, int64_t rows, int w, int planes,
+                                                          const long long* __restrict__ parts,
+                                                          unsigned long long* __restrict__ limbs) {
+  const int lane = threadIdx.x & 31;
+  const int64_t v = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (v >= count) return;
+  __int128 acc = 0;
+  for (int p = 0; p < planes; ++p) {
+    long long q = 0;
+    for (int64_t r = lane; r < rows; r += 32) q += parts[((int64_t)p * rows + r) * count + v];
+    for (int o = 16; o; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    acc += (__int128)q << (w * p);
+  }
+  if (lane != 0) return;
+  limbs[v * 3] = (unsigned long long)(acc & 0xFFFFFF);
+  limbs[v * 3 + 1] = (unsigned long long)((acc >> 24) & 0xFFFFFF);
+  limbs[v * 3 + 2] = (unsigned long long)(long long)(acc >> 48);
+}
+
+// Digit width, planes and scale; false when the form does not apply.
+bool plane_scale(const DevInstance& I, bool exact, int* w, int* planes, int* shift) {
+  int lg = 0;
+  while (((int64_t)1 << lg) < I.n) ++lg;
+  *w = std::min(12, 23 - lg);
+  if (*w < 9) return false;  // n <= 16384
+  if (exact || I.j_nonzeros == 0) {
+    *shift = 0;
+    int bits = 1;
+    while (std::ldexp(1.0, bits) <= I.j_absmax) ++bits;
+    *planes = (bits + 1 + *w - 1) / *w;
+    return true;
+  }
+  for (*planes = 4; *planes <= 7; ++*planes)
+    if (scale_for(I, std::min(58, *w * *planes - 2), shift)) return true;
+  return false;
+}
+
+template <typename T>
+int split_launch(ising_ctx* ctx, const DevInstance& I, int64_t ld, int shift, int w, int planes,
+                 uint16_t* out) {
+  const dim3 grid((unsigned)std::min<int64_t>((I.n + 1023) / 1024, 64), (unsigned)std::min<int64_t>(I.n, 65535));
+  split_digits_kernel<T><<<grid, 256, 0, ctx->stream>>>(I.J.as<T>(), I.n, ld, shift,
+                                                        std::ldexp(1.0, shift), w, planes, out);
+  ISING_CUDA(ctx, cudaGetLastError());
+  return ISING_OK;
 }
 
 // --------------------------------------------------------------- packed form
@@ -468,6 +566,32 @@ int read_odd(ising_ctx* ctx, const DevMem& odd, bool* ok) {
   return ISING_OK;
 }
 
+// The limbs of s^T I s by the planes form (spins known to be +-1 or the result
+// is thrown away by the caller).
+int plane_limbs(ising_ctx* ctx, const DevInstance& inst, int w, int planes, int shift,
+                const int8_t* spins, int64_t count, unsigned long long* limbs) {
+  const int64_t n = inst.n, ld = (n + 63) / 64 * 64, rows = 4 * ((n + 127) / 128);
+  DevMem P, S, parts;
+  ISING_TRY(dev_alloc(ctx, P, (size_t)planes * n * ld * 2));
+  ISING_TRY(dev_alloc(ctx, S, (size_t)count * ld * 2));
+  ISING_TRY(dev_alloc(ctx, parts, (size_t)planes * rows * count * 8));
+  uint16_t* out = P.as<uint16_t>();
+  switch (inst.j_dtype) {
+    case ISING_F64: ISING_TRY(split_launch<double>(ctx, inst, ld, shift, w, planes, out)); break;
+    case ISING_F32: ISING_TRY(split_launch<float>(ctx, inst, ld, shift, w, planes, out)); break;
+    case ISING_I8: ISING_TRY(split_launch<int8_t>(ctx, inst, ld, shift, w, planes, out)); break;
+    default: ISING_TRY(split_launch<int32_t>(ctx, inst, ld, shift, w, planes, out)); break;
+  }
+  spins_f16_kernel<<<pack_grid(ctx, (count * ld + 31) / 32), 256, 0, ctx->stream>>>(spins, count, n, ld,
+                                                                                  S.as<uint16_t>());
+  ISING_CUDA(ctx, cudaGetLastError());
+  ISING_TRY(tc_plane_energies(ctx, n, ld, count, out, planes, S.p, parts.as<long long>()));
+  join_digits_kernel<<<ceil_div_i(count, 8), 256, 0, ctx->stream>>>(count, rows, w, planes,
+                                                                    parts.as<long long>(), limbs);
+  ISING_CUDA(ctx, cudaGetLastError());
+  return ISING_OK;
+}
+
 int energy_fixed(ising_ctx* ctx, const DevInstance& inst, bool exact, int shift,
                  const int8_t* spins, int64_t count, double* E, int64_t* Q, int64_t* H, bool* ok) {
   const int64_t n = inst.n, words = (n + 31) / 32;
@@ -483,7 +607,15 @@ int energy_fixed(ising_ctx* ctx, const DevInstance& inst, bool exact, int shift,
   ISING_CUDA(ctx, cudaGetLastError());
   const uint32_t* bw = bits.as<uint32_t>();
   unsigned long long* L = limbs.as<unsigned long long>();
-  switch (inst.j_dtype) {
+  int w = 0, planes = 0, pshift = 0, rc = ISING_ENOMEM;  // (or no room for the planes)
+  // (from 16 vectors and 2^28 coupling-vectors on: n = 4096 takes 35 us per four
+  // vectors in the fixed form and about 200 us for 256 in planes)
+  if (count >= 16 && (double)n * (double)n * (double)count >= 268435456.0 &&
+      plane_scale(inst, exact, &w, &planes, &pshift))
+    rc = plane_limbs(ctx, inst, w, planes, pshift, spins, count, L);
+  if (rc == ISING_OK) shift = pshift;
+  else if (rc != ISING_ENOMEM) return rc;
+  else switch (inst.j_dtype) {
     case ISING_F64: ISING_TRY(fixed_launch_t<double>(ctx, inst, shift, bw, words, count, L)); break;
     case ISING_F32: ISING_TRY(fixed_launch_t<float>(ctx, inst, shift, bw, words, count, L)); break;
     case ISING_I8: ISING_TRY(fixed_launch_t<int8_t>(ctx, inst, shift, bw, words, count, L)); break;
@@ -536,7 +668,8 @@ int energy_packed(ising_ctx* ctx, const DevInstance& inst, bool exact, const int
 }  // namespace
 
 // Which form runs: the fixed form for every dense J that one scale holds (at
-// n = 4096 FP32: 256 vectors 23.5 -> 2.5 ms; one vector of n = 1000: 166 -> 6.4 us),
+// n = 4096 FP32: 256 vectors 23.5 ms in the general form, 2.5 in the fixed, 0.2
+// in planes; one vector of n = 1000: 166 -> 6.4 us),
 // the packed form for 8 or more vectors of a CSR instance (below that its lanes
 // are as idle as the general form's), the general form otherwise and whenever
 // a spin is not +-1.

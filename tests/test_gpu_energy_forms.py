@@ -42,6 +42,42 @@ def test_dense_float(gpu_ctx, dtype, n, count):
     _check_float(gpu_ctx, inst, _spins(count, n, n + count))
 
 
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("n,count", [(520, 1000), (1025, 300), (2050, 70), (4100, 17)])
+def test_dense_many_vectors(gpu_ctx, dtype, n, count):
+    """Digits in planes: 12 bits each up to n = 2048, 11 and 10 beyond (a
+    sampled subset of the vectors is checked)."""
+    inst = synth.sk_dense(n, n, 1.0, dtype, h_std=0.3)
+    s = _spins(count, n, n + count)
+    E = api.energy(gpu_ctx, inst, s)
+    pick = np.unique(np.linspace(0, count - 1, 12).astype(int))
+    cq, ch = ising.coefficients(inst.j_scale, inst.convention)
+    J, h = np.asarray(inst.J, np.longdouble), np.asarray(inst.h, np.longdouble)
+    x = s[pick].astype(np.longdouble)
+    ref = cq * ((x @ J) * x).sum(1) + ch * (x @ h)
+    bound = EPS * (24 * abs(cq) * np.abs(J).sum() + (n + 8) * np.abs(h).sum())
+    assert np.all(np.abs(E[pick] - ref) <= float(bound))
+    # one vector at a time takes the fixed form: the same integers up to the scale
+    one = np.array([api.energy(gpu_ctx, inst, s[k:k + 1])[0] for k in pick[:3]])
+    assert np.all(np.abs(one - E[pick[:3]]) <= float(bound))
+
+
+@pytest.mark.parametrize("dtype", [np.int8, np.int32, np.float32])
+def test_dense_integers_many_vectors(gpu_ctx, dtype):
+    n, count = 1030, 260
+    inst = synth.random_sparse_instance(n, 2, p=0.3, kind="int", h="int", layout="dense",
+                                        jmax=100 if dtype == np.int8 else 100000)
+    inst.J = inst.J.astype(dtype)
+    s = _spins(count, n, 1)
+    ref = synth.Instance(n=n, layout="dense", J=inst.J.astype(np.int32), h=inst.h,
+                         j_scale=inst.j_scale, convention=inst.convention)
+    E, Q, H = api.energy(gpu_ctx, inst, s, exact_parts=True)
+    Eo, Qo, Ho = ising.energy_exact(ref, s.T)
+    np.testing.assert_array_equal(Q, Qo)
+    np.testing.assert_array_equal(H, Ho)
+    np.testing.assert_array_equal(E, Eo)
+
+
 @pytest.mark.parametrize("scale", [1e-30, 1.0, 3e28])
 def test_dense_float_scales(gpu_ctx, scale):
     inst = synth.sk_dense(260, 5, 1.0, np.float32)
