@@ -558,9 +558,9 @@ int energy_general(ising_ctx* ctx, const DevInstance& inst, bool exact, const in
 }
 
 // Whether every spin was +-1; `odd` is the flag the packing kernel raised.
-int read_odd(ising_ctx* ctx, const DevMem& odd, bool* ok) {
+int read_odd(ising_ctx* ctx, const unsigned int* odd, bool* ok) {
   unsigned int o = 0;
-  ISING_CUDA(ctx, cudaMemcpyAsync(&o, odd.p, 4, cudaMemcpyDeviceToHost, ctx->stream));
+  ISING_CUDA(ctx, cudaMemcpyAsync(&o, odd, 4, cudaMemcpyDeviceToHost, ctx->stream));
   ISING_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   *ok = o == 0;
   return ISING_OK;
@@ -595,18 +595,14 @@ int plane_limbs(ising_ctx* ctx, const DevInstance& inst, int w, int planes, int 
 int energy_fixed(ising_ctx* ctx, const DevInstance& inst, bool exact, int shift,
                  const int8_t* spins, int64_t count, double* E, int64_t* Q, int64_t* H, bool* ok) {
   const int64_t n = inst.n, words = (n + 31) / 32;
-  DevMem bits, limbs;  // limbs [count][3], then the flag
-  ISING_TRY(dev_alloc(ctx, bits, (size_t)(count * words) * 4));
-  ISING_TRY(dev_alloc(ctx, limbs, (size_t)count * 24));
-  DevMem odd;
-  ISING_TRY(dev_alloc(ctx, odd, 4));
-  ISING_CUDA(ctx, cudaMemsetAsync(limbs.p, 0, (size_t)count * 24, ctx->stream));
-  ISING_CUDA(ctx, cudaMemsetAsync(odd.p, 0, 4, ctx->stream));
-  pack_rows_kernel<<<pack_grid(ctx, count * words), 256, 0, ctx->stream>>>(
-      spins, count, n, words, bits.as<uint32_t>(), odd.as<unsigned int>());
+  DevMem work;  // limbs [count][3], the flag (8 bytes), bits [count][words]
+  ISING_TRY(dev_alloc(ctx, work, (size_t)count * 24 + 8 + (size_t)(count * words) * 4));
+  ISING_CUDA(ctx, cudaMemsetAsync(work.p, 0, (size_t)count * 24 + 8, ctx->stream));
+  unsigned long long* L = work.as<unsigned long long>();
+  unsigned int* odd = reinterpret_cast<unsigned int*>(L + 3 * count);
+  uint32_t* bw = reinterpret_cast<uint32_t*>(odd + 2);
+  pack_rows_kernel<<<pack_grid(ctx, count * words), 256, 0, ctx->stream>>>(spins, count, n, words, bw, odd);
   ISING_CUDA(ctx, cudaGetLastError());
-  const uint32_t* bw = bits.as<uint32_t>();
-  unsigned long long* L = limbs.as<unsigned long long>();
   int w = 0, planes = 0, pshift = 0, rc = ISING_ENOMEM;  // (or no room for the planes)
   // (from 16 vectors and 2^28 coupling-vectors on: n = 4096 takes 35 us per four
   // vectors in the fixed form and about 200 us for 256 in planes)
@@ -662,17 +658,18 @@ int energy_packed(ising_ctx* ctx, const DevInstance& inst, bool exact, const int
                                                       0, E, nullptr, nullptr);
   }
   ISING_CUDA(ctx, cudaGetLastError());
-  return read_odd(ctx, odd, ok);
+  return read_odd(ctx, odd.as<unsigned int>(), ok);
 }
 
 }  // namespace
 
 // Which form runs: the fixed form for every dense J that one scale holds (at
 // n = 4096 FP32: 256 vectors 23.5 ms in the general form, 2.5 in the fixed, 0.2
-// in planes; one vector of n = 1000: 166 -> 6.4 us),
-// the packed form for 8 or more vectors of a CSR instance (below that its lanes
-// are as idle as the general form's), the general form otherwise and whenever
-// a spin is not +-1.
+// in planes; one vector of n = 1000: 166 -> 6.4 us;
+// but small integer ones, whose general form takes fewer launches: n = 121, 51
+// vectors 99 against 109 us per call), the packed form for 8 or more vectors of
+// a CSR instance (below that its lanes are as idle as the general form's), the
+// general form otherwise and whenever a spin is not +-1.
 int energy_device(ising_ctx* ctx, const DevInstance& inst, const int8_t* spins, int64_t count,
                   double* E, int64_t* Q, int64_t* H) {
   if (count <= 0) return ISING_OK;
@@ -681,7 +678,8 @@ int energy_device(ising_ctx* ctx, const DevInstance& inst, const int8_t* spins, 
   bool ok = false;
   int shift = 0;
   if (inst.layout == ISING_LAYOUT_DENSE) {
-    if (fixed_scale(inst, exact, &shift))
+    const double terms = (double)inst.n * (double)inst.n * (double)count;
+    if (!(exact && terms < 2097152.0) && fixed_scale(inst, exact, &shift))
       ISING_TRY(energy_fixed(ctx, inst, exact, shift, spins, count, E, Q, H, &ok));
   } else if (count >= 8) {
     ISING_TRY(energy_packed(ctx, inst, exact, spins, count, E, Q, H, &ok));
