@@ -176,6 +176,25 @@ struct ResLayout {
   static constexpr int kEpi = 4 * kParts;
 };
 
+// Sum over the 32 lanes of each of 4 columns, by the tree of column_sums8;
+// afterwards the lanes with bits b4 b3 hold the total of column 2 b4 + b3.
+template <typename T>
+__device__ __forceinline__ T column_sums4(T (&x)[4], int lane) {
+#pragma unroll
+  for (int o = 16, len = 2; o >= 8; o >>= 1, len >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int j = 0; j < len; ++j) {
+      T send = up ? x[j] : x[j + len];
+      T keep = up ? x[j + len] : x[j];
+      x[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  T y = x[0] + __shfl_xor_sync(0xffffffffu, x[0], 4);
+  y = y + __shfl_xor_sync(0xffffffffu, y, 2);
+  return y + __shfl_xor_sync(0xffffffffu, y, 1);
+}
+
 // Sum over the 32 lanes of each of 8 columns; afterwards lanes l, l^1, l^2,
 // l^3 hold the total of column 4 b4 + 2 b3 + b2 (bits of l).
 template <typename T>
@@ -1873,8 +1892,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
   constexpr int kBK = Lay::kBK;
   constexpr int esize = FP8 ? 1 : 2;
   constexpr uint32_t kTmemCols = 4 * BN;
-  constexpr int kCols = BN / 4;  // columns of one epilogue warp (8, 16 or 32)
-  constexpr int kWords = BN / 32;
+  constexpr int kCols = BN / 4;  // columns of one epilogue warp (4, 8, 16 or 32)
+  constexpr int kChunk = kCols < 8 ? kCols : 8;  // columns per TMEM read
+  constexpr int kWords = (BN + 31) / 32;
   const TcArgs& P = R.P;
   const int nk = P.nk, nkt = P.nk * P.planes;
   extern __shared__ uint8_t smem_raw[];
@@ -1967,9 +1987,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
         bm[j] = __float_as_uint(ok ? P.m[idx] : 0.f);
         c[j] = __float_as_uint(ok ? P.v[idx] : 0.f);
       }
-      tc::tmem_st8(t_th + c0, a);
-      tc::tmem_st8(t_m + c0, bm);
-      tc::tmem_st8(t_v + c0, c);
+      tc::tmem_st_cols(t_th + c0, a);
+      tc::tmem_st_cols(t_m + c0, bm);
+      tc::tmem_st_cols(t_v + c0, c);
     }
     tc::tmem_wait_st();
   }
@@ -1990,7 +2010,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     const float* pf = part_f + slot * 4 * BN;
 #pragma unroll
     for (int w = 0; w < kWords; ++w) {
-      const int b = 32 * w + lane;
+      const int b = min(32 * w + lane, BN - 1);  // (lanes past BN repeat the last)
       double E;
       if (INT_E) {
         const long long qs = (long long)pq[b] + pq[2 * BN + b] + pq[BN + b] + pq[3 * BN + b];
@@ -2000,8 +2020,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
         E = ((0.0 + (double)pf[b]) + (0.0 + (double)pf[2 * BN + b])) +
             ((0.0 + (double)pf[BN + b]) + (0.0 + (double)pf[3 * BN + b]));
       }
-      const bool better = E < bE[b] && n0 + b < P.B;
-      lE[b] = E;
+      const bool own = 32 * w + lane < BN;
+      const bool better = own && E < bE[b] && n0 + b < P.B;
+      if (own) lE[b] = E;
       if (better) {
         bE[b] = E;
         bT[b] = t0 + e + 1;
@@ -2051,7 +2072,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
       }
       __syncwarp();
       if (s >= 1) track(s - 1);
-    } else {
+    } else if (epi) {
       const float2 bcs = bc;
       if (!last) bc = P.bias[t + 1];  // used by the next step
       if (s >= 2) {
@@ -2070,10 +2091,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
 #pragma unroll 1
         for (int c0 = 0; c0 < kCols; c0 += kChunk) {
           uint32_t r[kChunk], th[kChunk], mm[kChunk], vv[kChunk];
-          tc::tmem_ld8(t_acc + c0, r);
-          tc::tmem_ld8(t_th + c0, th);
-          tc::tmem_ld8(t_m + c0, mm);
-          tc::tmem_ld8(t_v + c0, vv);
+          tc::tmem_ld_cols(t_acc + c0, r);
+          tc::tmem_ld_cols(t_th + c0, th);
+          tc::tmem_ld_cols(t_m + c0, mm);
+          tc::tmem_ld_cols(t_v + c0, vv);
           tc::tmem_wait_ld();
           int eq[kChunk];
           float ef[kChunk];
@@ -2095,9 +2116,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
           }
           cur_bits |= pos_bits << c0;
           if (!last) {
-            tc::tmem_st8(t_th + c0, th);
-            tc::tmem_st8(t_m + c0, mm);
-            tc::tmem_st8(t_v + c0, vv);
+            tc::tmem_st_cols(t_th + c0, th);
+            tc::tmem_st_cols(t_m + c0, mm);
+            tc::tmem_st_cols(t_v + c0, vv);
           }
           const int bl0 = part * kCols + c0;  // local restart of column j = 0
           if (row_ok) {
@@ -2137,8 +2158,13 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
               ph[q * BN + bl0 + lane] = hv;
             }
           } else {
-            const float te = column_sums8(ef, lane);
-            if ((lane & 3) == 0) pf[q * BN + bl0 + column_of_lane(lane)] = te;
+            if constexpr (kChunk == 8) {
+              const float te = column_sums8(ef, lane);
+              if ((lane & 3) == 0) pf[q * BN + bl0 + column_of_lane(lane)] = te;
+            } else {
+              const float te = column_sums4(ef, lane);
+              if ((lane & 7) == 0) pf[q * BN + bl0 + ((lane >> 3) & 1) + 2 * (lane >> 4)] = te;
+            }
           }
         }
         tc::tmem_wait_st();
@@ -2550,10 +2576,13 @@ int tc_setup(ising_ds* ds) {
   // (a tensor-memory kernel holds its SM alone): two groups of GN restarts
   // per CTA, 64 each, or 32 when B <= 64
   // small form: n <= 128, every CTA self-contained (no co-residency needed);
-  // the narrowest block of restarts (32, 64 or 128) that still fits one wave
+  // the narrowest block of restarts (16, the narrowest MMA of 128 rows, to
+  // 128) that still fits one wave: a step's epilogue is bound by instruction
+  // issue (100 spins, 64 restarts, 1000 steps: 3.23 ms with blocks of 32,
+  // 2.28 with 16)
   if (!(ds->p.flags & (ISING_DS_STREAMING | ISING_DS_CONVERGE)) && !ds->relaxed() && ds->n <= kBM) {
     int bn = 128;
-    for (int c : {32, 64})
+    for (int c : {16, 32, 64})
       if (ceil_div_i(ds->B, c) <= ctx->sm_count) {
         bn = c;
         break;
@@ -2797,7 +2826,9 @@ int tc_run_resident(ising_ds* ds, int64_t steps) {
     sa.cq = ds->inst.cq;
     sa.chs = ds->inst.ch * std::ldexp(1.0, -ds->h_shift);
     return st->gn == 128 ? small_launch_bn<128>(ds, st, sa)
-                         : (st->gn == 64 ? small_launch_bn<64>(ds, st, sa) : small_launch_bn<32>(ds, st, sa));
+                         : (st->gn == 64   ? small_launch_bn<64>(ds, st, sa)
+                            : st->gn == 32 ? small_launch_bn<32>(ds, st, sa)
+                                           : small_launch_bn<16>(ds, st, sa));
   }
   ISING_CUDA(ds->ctx, cudaMemsetAsync(st->gsync.p, 0, gsync_bytes(ds, st), ds->ctx->stream));
   TcResArgs r;
