@@ -180,7 +180,7 @@ def traffic_for(kernel: str, src_file: str, workload: str):
 
 
 def launches_per_solve(T: int, rounds: int, path: int, resident: bool, rowsum: bool,
-                       rowscale: bool) -> int:
+                       rowscale: bool, deferred: bool = False) -> int:
     """Kernels of one solve, as the ncu launch list of a solve shows them:
     instance checks (couplings twice, field once), pruning (dense->CSR 2,
     init 1, 7 per round incl. the final empty one, sum + reduced J + reduced
@@ -190,15 +190,16 @@ def launches_per_solve(T: int, rounds: int, path: int, resident: bool, rowsum: b
     (one launch when resident; on the streaming tensor-core path one launch
     per step, each also tracking its predecessor, plus one tracking launch
     for the last step; else step + track per step, plus the copy of improved
-    bit-packed spins on the sparse path), finish (energy-only step + track
-    (+ copy) + argmin), reconstruction (1), full-instance energy (2)."""
+    bit-packed spins on the sparse path, which the next step's tracking
+    launch makes when `deferred`: above 4096 spins), finish (energy-only step
+    + track (+ copy) + argmin), reconstruction (1), full-instance energy (2)."""
     per_step = 3 if path == 2 else 2
     if resident:
         steps = 1
     elif path == 1:
         steps = T + 1
     else:
-        steps = per_step * T
+        steps = (2 * T + 1 if T else 0) if deferred else per_step * T
     setup = 4 + (1 if rowsum else 0) + (1 if rowscale else 0)
     return 3 + 3 + 7 * (rounds + 1) + 3 + setup + steps + per_step + 1 + 1 + 2
 
@@ -808,7 +809,8 @@ def main():
                     "d2h_bytes_per_step": int(inst.n) + 8, "solves": e2e_k},
             "gpu_launches": launches_per_solve(
                 T, rounds, path, bool(last["resident"]), path == 1 and bool(inst.integer),
-                path == 1 and not inst.integer and prec in (2, 4)) * a.steps,
+                path == 1 and not inst.integer and prec in (2, 4),
+                path == 2 and n_red > 4096) * a.steps,
             "roofline": roof, "clocks": clk,
             "best_energy": float(last["best_energy"].item())}
     if name.startswith("table2"):

@@ -160,7 +160,7 @@ struct TrackArgs {
   double* last_E;
   long long* counters;
   int64_t bs_ld;
-  uint8_t* improved;
+  uint8_t* improved;  // [2][B], slot t mod 2
   int64_t T;
   double* conv_ring;
   double* conv_init;
@@ -168,7 +168,7 @@ struct TrackArgs {
   unsigned long long* conv_count;
   int* live32;  // live restarts per block of 32 (convergence rule), or null
   // bit-packed spins: copy an improved restart's spins here (small n)
-  // instead of flagging it for track_bits_copy_kernel
+  // instead of flagging it for copy_improved_bits
   bool inline_bits;
   // track the step counters[0] names, without advancing the counter (the
   // last step of a run whose step launches tracked their predecessors)
@@ -179,7 +179,7 @@ struct TrackArgs {
 // partials of slot t % 2 (lane l adds rows l, l+32, ... in order, then a
 // fixed xor tree across lanes, so the sum is deterministic), strict <
 // against the best so far, copy of S_t for an improved restart (for
-// bit-packed spins a per-restart flag instead, which track_bits_copy_kernel
+// bit-packed spins a per-restart flag instead, which copy_improved_bits
 // reads). With the convergence rule (conv_step non-null) a stopped restart
 // is left alone, and steps t <= T feed the rule.
 template <int KIND>
@@ -233,8 +233,8 @@ __device__ __forceinline__ void track_restart(const TrackArgs& A, long long t, i
           dst[i] = ((bits[i * words + (b >> 5)] >> (b & 31)) & 1u) ? 1 : -1;
       }
     } else if (lane == 0) {
-      // bit-packed spins are copied by track_bits_copy_kernel
-      A.improved[b] = improved ? 1 : 0;
+      // copied by the next tracking launch (copy_improved_bits)
+      A.improved[(t & 1) * A.B + b] = improved ? 1 : 0;
     }
   } else if (improved) {
     copy_spin_row_dense<KIND>(A.best_s + b * A.bs_ld, A.spins[t % 3], A.n, A.ld, b, lane);
