@@ -126,18 +126,20 @@ typedef struct ising_ds_params {
  * resident tensor-core form, one launch runs many steps: kernel_ms / kernel_launches
  * is then the time per step). */
 #define ISING_DS_PROFILE 1
-/* params.flags: keep the tensor-core path's state in device memory between
- * steps (one launch per step) even when a resident form would fit. The
- * resident forms keep theta, m and v in tensor memory across a whole run in
+/* params.flags: keep the state in device memory between steps (one launch
+ * per step) even when a resident form would fit. The resident form of the
+ * sparse path runs a whole run of steps in one launch with the state of each
+ * block's restarts in shared memory (instances whose spins, state and one to
+ * eight restarts fit there). The tensor-core path's resident forms keep theta, m and v in tensor memory across a whole run in
  * one launch: for n <= 128 the small form (every CTA holds all of J and the
- * spins of its block of restarts in shared memory, no grid-wide barrier), for
- * larger n the grid-wide form, used when every 128 x BN tile gets its own SM
- * (one cooperative launch). */
+ * spins of its block of 16 to 128 restarts in shared memory, no grid-wide
+ * barrier), for larger n the grid-wide form (one cooperative launch), used
+ * when every tile of 128 spins and 16 to 128 restarts gets its own SM. */
 #define ISING_DS_STREAMING 2
 /* params.flags: skip the launch-shape autotuner and use the default shape.
  * The autotuner times the first steps of a run once per problem shape with
- * each candidate shape and keeps the fastest: on the sparse path one or two
- * slices of 128 restarts per warp, on the tensor cores' streaming form the
+ * each candidate shape and keeps the fastest: on the sparse path's launch-per-step form
+ * one or two slices of 128 restarts per warp, on the tensor cores' streaming form the
  * restart-tile width (64, 128, 224 or 256 restarts per tile); results do not
  * depend on the shape. Choices are cached per process and, when the
  * environment variable ISING_TUNE_CACHE names a file, across processes. */
@@ -218,8 +220,9 @@ int ising_selftest_waits(ising_ctx* ctx, int64_t limit_cycles, int32_t* gave_up)
  * `mem`). Writes E_out[count] (float64) and, if Q_out / H_out are not NULL
  * and the instance is integer, the exact parts Q = s^T J s and H = h^T s
  * (int64, E = cQ Q + cH H). Integer couplings accumulate in integers and
- * are exact; other couplings accumulate in FP64. Outputs are in memory
- * `mem`. */
+ * are exact; other couplings accumulate in FP64, or for spins of +-1 in fixed
+ * point of more bits (many vectors of a dense instance: as exact FP16 digits
+ * of the couplings on the tensor cores). Outputs are in memory `mem`. */
 int ising_energy(ising_ctx* ctx, const ising_instance* inst, const int8_t* spins,
                  int64_t count, double* E_out, int64_t* Q_out, int64_t* H_out, int mem);
 
@@ -381,8 +384,9 @@ int ising_ds_last_energies(ising_ds* ds, double* E, int mem);
  * tensor-core forms count B per step). Without ISING_DS_CONVERGE this is
  * B x steps; with it, tiles and slices whose restarts have all stopped are
  * skipped (early retirement: their results are final, their state is left
- * where it stopped), so it falls below B x steps. The resident tensor-core
- * forms keep every restart running. Synchronises the session's stream. */
+ * where it stopped), so it falls below B x steps; the resident sparse form
+ * counts in the same slices of 128 restarts. The resident tensor-core forms
+ * keep every restart running. Synchronises the session's stream. */
 int ising_ds_work(ising_ds* ds, int64_t* restart_steps);
 /* Launch shape of the tensor-core streaming form set by hand: 64, 128, 224
  * or 256 restarts per tile; pair = 1 runs the tiles over clusters of two
@@ -421,7 +425,8 @@ int ising_ds_destroy(ising_ds* ds);
  * form (no grid barrier shared with other requests' kernels), except
  * instances of at most 128 spins without ISING_DS_CONVERGE or
  * ISING_DS_RELAXED, whose small resident form has none either and runs a
- * whole chunk of steps in one launch. The paper has no counterpart.
+ * whole chunk of steps in one launch; sparse requests that fit take the
+ * resident sparse form, whose blocks do not wait on one another. The paper has no counterpart.
  * The requests' streams reach the device through the context's hardware
  * work queues (8 unless the environment variable CUDA_DEVICE_MAX_CONNECTIONS,
  * read when the process creates its CUDA context, says more): with more

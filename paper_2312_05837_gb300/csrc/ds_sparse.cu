@@ -1,4 +1,6 @@
-// K2s: fused domain-selection step (Sec. III-B) for CSR couplings.
+// K2s: fused domain-selection step (Sec. III-B) for CSR couplings, one launch
+// per step (instances that fit shared memory take the resident form,
+// ds_sparse_res.cu).
 //
 // Layout: state theta, m, v is [n][Bp] (restarts contiguous, Bp a multiple of
 // 128); spins are bit-packed [n][Bp/32] words (bit set = +1). A block covers

@@ -12,9 +12,11 @@
 // contiguous; kind::f16 takes both operands in one type). Both operands are
 // K-major, so one TMA box of 128 bytes (a k-block: 128 E4M3 or 64 16-bit
 // elements) x rows fills a 128-byte swizzled shared-memory tile that
-// tcgen05.mma reads directly. A thread issues one tcgen05.mma only every ~110
-// cycles and one TMA copy every ~250 whatever their sizes, which shapes the
-// kernels below.
+// tcgen05.mma reads directly. A thread chosen by elect.sync issues an M-128
+// tcgen05.mma every 53 cycles at N 64, 64 at N 128 and 128 at N 256 (74 at
+// N 64 when a lane test chooses it); a producer iteration (wait, expect, copy)
+// costs 400 to 640 cycles whatever it copies and 25 to 80 per further copy:
+// measured by probe kernels, this shapes the kernels below.
 //
 // Streaming form (tc_step_kernel): one persistent CTA per SM, warp-specialised:
 //   warps 0, 2 TMA producers of the J and the S tiles of a STAGES-deep ring
@@ -1135,12 +1137,14 @@ __global__ void row_absmax_kernel(const void* J, int dt, int64_t n, float* scale
 // Resident form: when every tile of the problem fits one CTA per SM, each CTA
 // keeps its tile of theta, m, v in tensor memory for a whole run of steps, so
 // a step moves only the J / S tiles (TMA) and the new spins and energy
-// partials (global stores). A CTA holds two groups of GN restarts, each with
-// its own tensor-memory block (accumulator, theta, m, v: columns
-// [4 GN g, 4 GN (g + 1))), and the tensor cores alternate between them: while
-// the epilogue warps update group 0 from its accumulator, the MMAs of group 1
-// run, and the other way round, so the MMA stream (paced by one thread's issue
-// rate) and the epilogue (bound by instruction issue) overlap. Step t + 1 of
+// partials (global stores). A CTA holds one group of GN = 16, 32 or 64
+// restarts, or two of 64, each with its own tensor-memory block (accumulator,
+// theta, m, v: columns [4 GN g, 4 GN (g + 1))). With two groups the tensor
+// cores alternate between them: while the epilogue warps update group 0 from
+// its accumulator, the MMAs of group 1 run, and the other way round. One
+// group is taken where every tile then has its own SM: nothing overlaps, but
+// the step's chain (copies, MMAs, epilogue, column barrier) is shorter
+// (1000 spins, 1024 restarts: 19.5 -> 14.9 us per step). Step t + 1 of
 // a group needs S_t of all rows, i.e. the output of every m-tile of the same
 // restarts, so the CTAs of one group's column pass a barrier between steps
 // (an arrival counter per group and column; the cooperative launch keeps all
@@ -2579,9 +2583,6 @@ int tc_setup(ising_ds* ds) {
     }
   }
   st->nfull = (int)(ds->n / (st->fp8 ? 128 : 64));
-  // resident form when every (128 x 2 GN) tile gets its own co-resident CTA
-  // (a tensor-memory kernel holds its SM alone): two groups of GN restarts
-  // per CTA, 64 each, or 32 when B <= 64
   // small form: n <= 128, every CTA self-contained (no co-residency needed);
   // the narrowest block of restarts (16, the narrowest MMA of 128 rows, to
   // 128) that still fits one wave: a step's epilogue is bound by instruction
