@@ -173,7 +173,7 @@ __device__ __forceinline__ long long to_fixed(T x, int shift, double dscale) {
     const long long m = (long long)((((unsigned long long)mant << 38) + (1ull << (d - 1))) >> d);
     return (int)u < 0 ? -m : m;
   } else {
-    return (long long)x;
+    return (long long)x;  // (integer types are never scaled: whole_couplings)
   }
 }
 
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(256) energy_fixed_finish(
   }
 }
 
-// The binary scale of the fixed form: 0 and *b = 0 for exact integers; else
+// The binary scale of the fixed form: 0 for integer couplings; else
 // every J_ij becomes rint(J_ij 2^*shift) with b bits, b the most for which no
 // lane's sums overflow. Each rounding is off by at most 2^-(b + 1) 2^E
 // (|J| < 2^E), all of them together by no more than 16 2^-53 sum |J_ij|, which
@@ -323,9 +323,13 @@ bool scale_for(const DevInstance& I, int b, int* shift) {
   return *shift >= -120 && *shift <= 120;  // a float power of two; no result underflows
 }
 
-bool fixed_scale(const DevInstance& I, bool exact, int* shift) {
+// Integer couplings that the integer forms add as they are (scale 0): whatever
+// the fields, whose sum of a non-dyadic h stays in FP64.
+bool whole_couplings(const DevInstance& I) { return I.j_integer && I.j_absmax <= 2147483648.0; }
+
+bool fixed_scale(const DevInstance& I, int* shift) {
   *shift = 0;
-  if (exact || I.j_nonzeros == 0) return true;
+  if (whole_couplings(I) || I.j_nonzeros == 0) return true;
   const int64_t lane_terms = 4 * ((I.n + 1023) / 1024) + 4;
   int lg = 0;
   while (((int64_t)1 << lg) < lane_terms) ++lg;
@@ -424,12 +428,12 @@ __global__ void __launch_bounds__(256) join_digits_kernel(int64_t count, int64_t
 }
 
 // Digit width, planes and scale; false when the form does not apply.
-bool plane_scale(const DevInstance& I, bool exact, int* w, int* planes, int* shift) {
+bool plane_scale(const DevInstance& I, int* w, int* planes, int* shift) {
   int lg = 0;
   while (((int64_t)1 << lg) < I.n) ++lg;
   *w = std::min(12, 23 - lg);
   if (*w < 9) return false;  // n <= 16384
-  if (exact || I.j_nonzeros == 0) {
+  if (whole_couplings(I) || I.j_nonzeros == 0) {
     *shift = 0;
     int bits = 1;
     while (std::ldexp(1.0, bits) <= I.j_absmax) ++bits;
@@ -607,7 +611,7 @@ int energy_fixed(ising_ctx* ctx, const DevInstance& inst, bool exact, int shift,
   // (from 16 vectors and 2^28 coupling-vectors on: n = 4096 takes 35 us per four
   // vectors in the fixed form and about 200 us for 256 in planes)
   if (count >= 16 && (double)n * (double)n * (double)count >= 268435456.0 &&
-      plane_scale(inst, exact, &w, &planes, &pshift))
+      plane_scale(inst, &w, &planes, &pshift))
     rc = plane_limbs(ctx, inst, w, planes, pshift, spins, count, L);
   if (rc == ISING_OK) shift = pshift;
   else if (rc != ISING_ENOMEM) return rc;
@@ -679,7 +683,7 @@ int energy_device(ising_ctx* ctx, const DevInstance& inst, const int8_t* spins, 
   int shift = 0;
   if (inst.layout == ISING_LAYOUT_DENSE) {
     const double terms = (double)inst.n * (double)inst.n * (double)count;
-    if (!(exact && terms < 2097152.0) && fixed_scale(inst, exact, &shift))
+    if (!(exact && terms < 2097152.0) && fixed_scale(inst, &shift))
       ISING_TRY(energy_fixed(ctx, inst, exact, shift, spins, count, E, Q, H, &ok));
   } else if (count >= 8) {
     ISING_TRY(energy_packed(ctx, inst, exact, spins, count, E, Q, H, &ok));
