@@ -171,12 +171,23 @@ struct ResLayout {
   static constexpr uint32_t kA = kBM * kRowBytes;
   static constexpr uint32_t kB = GN * kRowBytes;
   static constexpr uint32_t kJ = 2 * kA;  // J tiles of a unit
-  static constexpr int kMaxSlots = 16;
   // epilogue warps: four per part of the group's columns, at least one chunk each
   static constexpr int kParts = GN >= 32 ? 4 : GN / 8;
   static constexpr int kCols = GN / kParts;
   static constexpr int kEpi = 4 * kParts;
 };
+
+// The resident form's barriers and words in shared memory, after its tiles.
+constexpr int kResSlots = 16;  // of each ring at most
+struct ResBars {
+  uint64_t sfull[kResSlots], sempty[kResSlots], jfull[kResSlots], jempty[kResSlots];
+  uint64_t rfull;  // the resident J tiles have landed
+  uint64_t acc_full[2], acc_empty[2], step_done[2], go[2];  // per restart group
+  uint64_t drain;
+  uint32_t tmem_slot;
+  int abort_flag;
+};
+constexpr size_t kResTail = (sizeof(ResBars) + 127) / 128 * 128;
 
 // Sum over the 32 lanes of each of 4 columns, by the tree of column_sums8;
 // afterwards the lanes with bits b4 b3 hold the total of column 2 b4 + b3.
@@ -1495,22 +1506,18 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t kS = two ? Lay::kB : 2 * Lay::kB;  // S tiles of a unit
   uint8_t* jring = smem + (uint32_t)ru * Lay::kJ;
   uint8_t* sring = jring + (uint32_t)nj * Lay::kJ;
-  uint64_t* sfull = reinterpret_cast<uint64_t*>(smem + R.bars);
-  uint64_t* sempty = sfull + Lay::kMaxSlots;
-  uint64_t* jfull = sempty + Lay::kMaxSlots;
-  uint64_t* jempty = jfull + Lay::kMaxSlots;
-  uint64_t* rfull = jempty + Lay::kMaxSlots;  // the resident J tiles have landed
-  uint64_t* acc_full = rfull + 1;       // [2], one per restart group
-  uint64_t* acc_empty = acc_full + 2;   // [2]
-  uint64_t* step_done = acc_empty + 2;  // [2]
-  uint64_t* go = step_done + 2;         // [2]
-  uint64_t* drain = go + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  ResBars* const bars = reinterpret_cast<ResBars*>(smem + R.bars);
+  uint64_t *const sfull = bars->sfull, *const sempty = bars->sempty;
+  uint64_t *const jfull = bars->jfull, *const jempty = bars->jempty;
+  uint64_t *const rfull = &bars->rfull, *const acc_full = bars->acc_full;
+  uint64_t *const acc_empty = bars->acc_empty, *const step_done = bars->step_done;
+  uint64_t *const go = bars->go, *const drain = &bars->drain;
+  uint32_t* const tmem_slot = &bars->tmem_slot;
+  volatile int* const abort_flag = &bars->abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < Lay::kMaxSlots; ++s) {
+    for (int s = 0; s < kResSlots; ++s) {
       tc::mbar_init(&sfull[s], 1);
       tc::mbar_init(&sempty[s], 1);
       tc::mbar_init(&jfull[s], 1);
@@ -2621,14 +2628,14 @@ int tc_setup(ising_ds* ds) {
       // shared memory: resident units, the J and the S ring, the barrier block
       const int64_t kJ = 2 * (int64_t)kBM * kRowBytes;
       const int64_t kS = (int64_t)gn * kRowBytes * (ds->planes == 2 ? 1 : 2);
-      const int64_t region = ((int64_t)ctx->smem_optin - 1024 - 512) / 1024 * 1024;
+      const int64_t region = ((int64_t)ctx->smem_optin - 1024 - (int64_t)kResTail) / 1024 * 1024;
       const int units = (ceil_div_i(ds->n, st->fp8 ? 128 : 64) * ds->planes + 1) / 2;
       // the split of the room between resident units and the two rings by the
       // time a phase's copies take: a ring moves its bytes per round trip
       // (about 2 us from L2 under load), both together at most 90 GB/s per SM
       int ns = 2, nj = 0, ru = -1;
       double best = 0.0;
-      for (int cs = 2; cs <= 16; ++cs)
+      for (int cs = 2; cs <= kResSlots; ++cs)
         for (int cj = 0; cj <= 8; ++cj) {
           const int64_t left = region - cs * kS - cj * kJ;
           const int cr = (int)std::min<int64_t>(units, left < 0 ? -1 : left / kJ);
@@ -2640,7 +2647,7 @@ int tc_setup(ising_ds* ds) {
         }
       int nb = 0;
       if (ru >= 0) {
-        const size_t bytes = (size_t)region + 512 + 1024;
+        const size_t bytes = (size_t)region + kResTail + 1024;  // + alignment slack
         if (gr == 2) ISING_TRY((resident_attr_bn<64, 2>(ds, st->fp8, bytes, &nb)));
         else if (gn == 64) ISING_TRY((resident_attr_bn<64, 1>(ds, st->fp8, bytes, &nb)));
         else if (gn == 32) ISING_TRY((resident_attr_bn<32, 1>(ds, st->fp8, bytes, &nb)));
