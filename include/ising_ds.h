@@ -183,9 +183,8 @@ typedef struct ising_ds_stats {
   int32_t operand_planes;   /* tensor-core path: operand planes of J per product (1 or 2;
                                the tensor cores execute that many products), else 1 */
   int32_t tile_restarts;    /* tensor-core streaming form: restarts per tile, else 0 */
-  int32_t tile_pair;        /* tensor-core streaming form: 0 one CTA per tile, 1 CTA pairs
-                               sharing spin tiles by multicast, 2 one MMA per CTA pair
-                               (see ising_ds_set_tiles); else 0 */
+  int32_t tile_pair;        /* tensor-core streaming form: 0 one CTA per tile, 2 one MMA
+                               per CTA pair (see ising_ds_set_tiles); else 0 */
 } ising_ds_stats;
 
 /* ------------------------------------------------------------------ context */
@@ -389,11 +388,10 @@ int ising_ds_last_energies(ising_ds* ds, double* E, int mem);
  * keep every restart running. Synchronises the session's stream. */
 int ising_ds_work(ising_ds* ds, int64_t* restart_steps);
 /* Launch shape of the tensor-core streaming form set by hand: 64, 128, 224
- * or 256 restarts per tile; pair = 1 runs the tiles over clusters of two
- * CTAs that share each spin tile (each loads half and multicasts it to
- * both; widths 224 and 256, more than 128 spins); pair = 2 as well, but
- * each CTA keeps its half and the pair's MMAs run as one (M 256 over the
- * two CTAs, cta_group::2). The autotuner leaves the
+ * or 256 restarts per tile; pair = 2 runs the tiles over clusters of two
+ * CTAs (widths 224 and 256, more than 128 spins): each CTA keeps half of the
+ * spin tile and the pair's MMAs run as one (M 256 over the two CTAs,
+ * cta_group::2). pair = 1 is accepted for the same. The autotuner leaves the
  * session alone afterwards. Results do not depend on the shape. ISING_ENOTSUP
  * on other forms, ISING_EINVAL for a shape the session cannot take. No
  * counterpart in the paper: a tuning control. */

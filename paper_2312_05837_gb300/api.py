@@ -529,9 +529,8 @@ class Session:
         return E
 
     def set_tiles(self, restarts_per_tile: int, pair: int = 0):
-        """Tensor-core streaming form: tile width and CTA pairs (0 none, 1
-        sharing spin tiles by multicast, 2 one MMA per pair; see
-        ising_ds_set_tiles)."""
+        """Tensor-core streaming form: tile width and CTA pairs (0 none, 2 one
+        MMA per pair, 1 the same; see ising_ds_set_tiles)."""
         self.ctx.check(self.ctx.lib.ising_ds_set_tiles(self.handle, int(restarts_per_tile),
                                                        int(pair)))
 

@@ -1320,7 +1320,7 @@ extern "C" int ising_ds_set_tiles(ising_ds* ds, int32_t restarts_per_tile, int32
   if (ds->path != ISING_PATH_TC || tc_is_resident(ds))
     return fail(ctx, ISING_ENOTSUP, "tile shapes apply to the tensor-core streaming form");
   if (pair < 0 || pair > 2) return fail(ctx, ISING_EINVAL, "pair must be 0, 1 or 2");
-  const int code = restarts_per_tile | (pair ? kTcPair : 0) | (pair == 2 ? kTcSplit : 0);
+  const int code = restarts_per_tile | (pair ? kTcPair : 0);  // (1 and 2 name one form)
   int cand[8];
   const int nc = tc_bn_candidates(ds, cand);
   bool ok = restarts_per_tile == 64 || restarts_per_tile == 128 || restarts_per_tile == 224 ||

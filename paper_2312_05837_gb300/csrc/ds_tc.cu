@@ -33,11 +33,9 @@
 //              new spin into S_{t+1}, and the energy of the input spins, summed
 //              over each warp's 32 spins by a butterfly across lanes into
 //              one partial row per warp (summed in fixed order afterwards).
-// The same roles run in clusters of two CTAs (tc_step_pair_kernel: each
-// loads half of the spin tile and multicasts it to both; tc_step_split_kernel:
-// the pair's MMAs issued as one, cta_group::2, M 256, each CTA holding its J
-// rows and half of the spin tile), shapes the autotuner times beside single
-// CTAs.
+// The same roles run in clusters of two CTAs (tc_step_split_kernel: the pair's
+// MMAs issued as one, cta_group::2, M 256, each CTA holding its J rows and half
+// of the spin tile), shapes the autotuner times beside single CTAs.
 // Tiles are numbered row tile by row tile (the restart tiles of one row tile
 // are consecutive), so one wave of persistent CTAs covers whole row tiles: a
 // J row tile is read from HBM about once per step and shared through L2 by
@@ -319,7 +317,6 @@ __device__ __noinline__ int balanced_tile(int total, int per_row, int groups, in
 template <int BN>
 struct OneInstance {
   static constexpr bool kGlobalMaps = false;  // kernel parameters
-  static constexpr bool kPair = false;
   static constexpr bool kSplit = false;
   static constexpr bool kFold = true;  // may track the previous step (TcArgs::fold)
   const TcArgs& P;  // the kernel's parameter
@@ -388,7 +385,6 @@ struct __align__(64) PackEntry {
 template <int BN>
 struct PackedInstances {
   static constexpr bool kGlobalMaps = true;  // copied to device memory by the host
-  static constexpr bool kPair = false;
   static constexpr bool kSplit = false;
   static constexpr bool kFold = true;  // may track every member's previous step (trk)
   __device__ int first() const { return blockIdx.x; }
@@ -465,21 +461,17 @@ struct PackedInstances {
 
 // Tiles of one instance for clusters of two CTAs: a cluster takes pair tile
 // (pm, nt), its CTA of rank r the row tile 2 pm + r of restart tile nt. Both
-// CTAs need the same spin tile: each loads one half of it and multicasts the
-// half to both (the J tiles are their own), so a CTA reads 30 instead of 44
-// KB per stage from L2 at tiles of 224 restarts. With an odd number of row
-// tiles the last pair's second tile lies past n (zero rows, nothing written).
-// SPLIT: instead of multicasting, each CTA keeps its half of the spin tile
-// and the first CTA issues the MMAs of the pair (cta_group::2, M 256): a
-// CTA's shared memory then holds and serves 30 instead of 44 KB per stage,
-// which is what limits the operand stream of single-CTA tiles (the tensor
-// cores read a stage as fast as TMA writes it, both through the SM's shared
-// memory).
-template <int BN, bool SPLIT = false>
+// CTAs need the same spin tile: each keeps one half of it, and the first CTA
+// issues the MMAs of the pair (cta_group::2, M 256), which read both halves
+// where they are. A CTA so loads, holds and serves 30 instead of 44 KB per
+// stage at tiles of 224 restarts, which is what limits the operand stream of
+// single-CTA tiles (the tensor cores read a stage as fast as TMA writes it,
+// both through the SM's shared memory). With an odd number of row tiles the
+// last pair's second tile lies past n (zero rows, nothing written).
+template <int BN>
 struct PairInstance {
   static constexpr bool kGlobalMaps = false;
-  static constexpr bool kPair = true;
-  static constexpr bool kSplit = SPLIT;
+  static constexpr bool kSplit = true;
   static constexpr bool kFold = true;
   const TcArgs& P;
   const CUtensorMap *A0, *A1, *A2, *J0, *J1, *J2;
@@ -490,13 +482,13 @@ struct PairInstance {
   // the CTA's j-th tile (row-tile-major order)
   __device__ int at(int j) const {
     const int per_row = (int)((P.B + 31) / 32);
-    if (SPLIT && P.balanced)
+    if (P.balanced)
       return balanced_tile((P.mtiles + 1) / 2 * per_row, per_row, stride(), first(), BN / 32, j);
     return first() + j * stride();
   }
   __device__ int total() const {
-    return SPLIT && P.balanced ? (P.mtiles + 1) / 2 * (int)((P.B + 31) / 32) * 16
-                               : (P.mtiles + 1) / 2 * P.ntiles;
+    return P.balanced ? (P.mtiles + 1) / 2 * (int)((P.B + 31) / 32) * 16
+                      : (P.mtiles + 1) / 2 * P.ntiles;
   }
   __device__ int* err() const { return P.err; }
   __device__ unsigned long long* trace() const { return P.trace; }
@@ -523,7 +515,7 @@ struct PairInstance {
     r.qpart = P.qpart;
     r.hpart = P.hpart;
     r.epart = P.epart;
-    if (SPLIT && P.balanced) {
+    if (P.balanced) {
       const int per_row = (int)((P.B + 31) / 32);
       r.mt = 2 * ((tl >> 4) / per_row) + (int)rank;
       r.n0 = (tl >> 4) % per_row * 32;
@@ -553,7 +545,7 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
   constexpr bool SPLIT = Src::kSplit;
   using Lay = TcLayout<BN, SPLIT>;
   constexpr int kBK = FP8 ? 128 : 64;  // elements per 128-byte row
-  static_assert(!Src::kPair || Lay::kKps == 1, "pair tiles take one k-block per stage");
+  static_assert(!SPLIT || Lay::kKps == 1, "pair tiles take one k-block per stage");
   // two J planes (every tile of the launch): stages of one k-block of both
   // planes and its spin tile, the MMAs taking the planes k-block by k-block
   const bool fused = !FP8 && src.fused();
@@ -578,9 +570,7 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       tc::mbar_init(&full[s], 2);  // the J and the S producer
-      // released by the MMA issuer of each CTA of a multicasting pair, or by
-      // the one issuer of a split pair (or of a single CTA)
-      tc::mbar_init(&empty[s], (Src::kPair && !SPLIT) ? 2 : 1);
+      tc::mbar_init(&empty[s], 1);  // the MMA issuer (a pair has one)
     }
     for (int b = 0; b < 2; ++b) {
       tc::mbar_init(&acc_full[b], 1);
@@ -598,7 +588,7 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
   }
   __syncthreads();
   // pairs: the partner's barriers are initialised before copies or commits target them
-  if (Src::kPair) tc::cluster_sync();
+  if (SPLIT) tc::cluster_sync();
   tc::fence_after_sync();
   if (threadIdx.x == 0) ISING_TRACE(0);
   const uint32_t tmem_base = *tmem_slot;
@@ -668,9 +658,6 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
             } else if constexpr (SPLIT) {
               if (lead) tc::tma_load_2d_hint(sb, T.B, &full[stage], kb * kBK, T.n0, pol);
               else tc::tma_load_2d_to_pair(sb, T.B, lead_full, kb * kBK, T.n0 + srows, pol);
-            } else if constexpr (Src::kPair) {
-              tc::tma_load_2d_mc(sb + src.rank * (srows / 2) * kRowBytes, T.B, &full[stage], kb * kBK,
-                                 T.n0 + (int)src.rank * (srows / 2), 0x3, pol);
             } else {
               tc::tma_load_2d_hint(sb, T.B, &full[stage], kb * kBK, T.n0, pol);
             }
@@ -700,10 +687,6 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
                 }
               } else if (jside) {
                 tc::tma_load_2d_hint(sa + u * Lay::kA, T.a(plane), &full[stage], kb * kBK, T.m0, pol);
-              } else if constexpr (Src::kPair) {
-                // this CTA's half of the spin tile, to both CTAs of the pair
-                tc::tma_load_2d_mc(sa + Lay::kA + src.rank * (srows / 2) * kRowBytes, T.B,
-                                   &full[stage], kb * kBK, T.n0 + (int)src.rank * (srows / 2), 0x3, pol);
               } else {
                 tc::tma_load_2d_hint(sa + Lay::kKps * Lay::kA + u * sbytes, T.B, &full[stage],
                                      kb * kBK, T.n0, pol);
@@ -716,10 +699,10 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
         }
       }
       if (jside) ISING_TRACE(2);
-      if (Src::kPair && ok && jside) {
-        // pairs: wait until both CTAs' MMA issuers have released every stage,
-        // so that no commit of the partner arrives on this CTA's barriers
-        // after it has left (the cluster barrier at the end follows)
+      if (SPLIT && ok && jside) {
+        // pairs: wait until the MMA issuer has released every stage, so that
+        // none of its commits arrives on the second CTA's barriers after it has
+        // left (the cluster barrier at the end follows)
         for (int q = 0; q < STAGES && ok; ++q) {
           ok = tc::mbar_wait(&empty[stage], phase ^ 1, abort_flag, kWaitCycles);
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
@@ -806,11 +789,9 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
               }
             }
           }
-          // the stage is free once this CTA's MMAs (and, for pairs, the
-          // partner's, whose spin half it also holds) have read it; a split
-          // pair's MMAs read both CTAs' stages
+          // the stage is free once the MMAs have read it (a pair's read both
+          // CTAs' stages)
           if constexpr (SPLIT) tc::mma_commit_pair_mc(&empty[stage], 0x3);
-          else if constexpr (Src::kPair) tc::mma_commit_mc(&empty[stage], 0x3);
           else tc::mma_commit(&empty[stage]);
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
@@ -987,7 +968,7 @@ __device__ __forceinline__ void step_tiles(const Src& src) {
   __syncthreads();
   // pairs: neither CTA leaves while the other may still copy into its shared
   // memory or arrive on its barriers
-  if (Src::kPair) tc::cluster_sync();
+  if (SPLIT) tc::cluster_sync();
   if (threadIdx.x == 0) ISING_TRACE(7);
   if constexpr (MODE == kModeUpdate && Src::kFold) src.advance_step();
   if (warp == 1) {
@@ -1012,23 +993,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   step_tiles<BN, MODE, INT_E, FP8>(src);
 }
 
-// The same over clusters of two CTAs sharing each spin tile (PairInstance).
-template <int BN, int MODE, bool INT_E, bool FP8>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-    tc_step_pair_kernel(const __grid_constant__ CUtensorMap tmA0,
-                        const __grid_constant__ CUtensorMap tmA1,
-                        const __grid_constant__ CUtensorMap tmA2,
-                        const __grid_constant__ WidthMaps tmBh,
-                        const __grid_constant__ CUtensorMap tmJ2_0,
-                        const __grid_constant__ CUtensorMap tmJ2_1,
-                        const __grid_constant__ CUtensorMap tmJ2_2,
-                        const __grid_constant__ TcArgs P) {
-  const PairInstance<BN> src{P,       &tmA0,   &tmA1, &tmA2, &tmJ2_0,
-                             &tmJ2_1, &tmJ2_2, &tmBh, tc::cluster_rank()};
-  step_tiles<BN, MODE, INT_E, FP8>(src);
-}
-
-// The same with the MMAs of each pair issued as one (cta_group::2, M 256).
+// The same over clusters of two CTAs, the MMAs of each pair issued as one (PairInstance).
 template <int BN, int MODE, bool INT_E, bool FP8>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     tc_step_split_kernel(const __grid_constant__ CUtensorMap tmA0,
@@ -1039,8 +1004,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                          const __grid_constant__ CUtensorMap tmJ2_1,
                          const __grid_constant__ CUtensorMap tmJ2_2,
                          const __grid_constant__ TcArgs P) {
-  const PairInstance<BN, true> src{P,       &tmA0,   &tmA1, &tmA2, &tmJ2_0,
-                                   &tmJ2_1, &tmJ2_2, &tmBh, tc::cluster_rank()};
+  const PairInstance<BN> src{P,       &tmA0,   &tmA1, &tmA2, &tmJ2_0,
+                             &tmJ2_1, &tmJ2_2, &tmBh, tc::cluster_rank()};
   step_tiles<BN, MODE, INT_E, FP8>(src);
 }
 
@@ -2251,8 +2216,7 @@ struct TcState {
   CUtensorMap J2[3], S2[3];
   CUtensorMap SP[3];  // streaming kernel: the spin slots' views of two k-blocks, boxes of BN restarts
   WidthMaps Bh[3];    // pair tiles: the spin slots, boxes of half the widths
-  bool pair = false;  // streaming kernel over clusters of two CTAs sharing spin tiles
-  bool split = false; // ... whose MMAs run as one per pair (cta_group::2)
+  bool pair = false;  // streaming kernel over clusters of two CTAs (one MMA per pair)
   int nfull = 0;      // k-blocks lying wholly below column n (0 in the small form)
   CUtensorMap Bx[2];  // relaxed mode: one per slot of x = sin(theta), boxes of BN restarts
   int BN = 128;
@@ -2334,7 +2298,7 @@ int launch_bn(ising_ds* ds, TcState* st, const TcArgs& a, const CUtensorMap& mB,
               const CUtensorMap& mS2, const WidthMaps& mBh) {
   const size_t smem = TcLayout<BN>::kBytes;
   if constexpr (BN >= 192) {
-    if (st->pair && st->split) {
+    if (st->pair) {
       auto kern = tc_step_split_kernel<BN, MODE, INT_E, FP8>;
       const size_t ssmem = TcLayout<BN, true>::kBytes;
       static bool attr_set = false;  // per instantiation
@@ -2348,23 +2312,6 @@ int launch_bn(ising_ds* ds, TcState* st, const TcArgs& a, const CUtensorMap& mB,
       kern<<<2 * clusters, kThreads, ssmem, ds->ctx->stream>>>(st->A[0], st->A[1], st->A[2], mBh,
                                                                st->J2[0], st->J2[1], st->J2[2],
                                                                a);
-      ISING_CUDA(ds->ctx, cudaGetLastError());
-      return ISING_OK;
-    }
-    if (st->pair) {
-      auto kern = tc_step_pair_kernel<BN, MODE, INT_E, FP8>;
-      static bool attr_set = false;  // per instantiation
-      if (!attr_set) {
-        ISING_CUDA(ds->ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem));
-        attr_set = true;
-      }
-      // one cluster of two CTAs per pair of SMs, at most one per pair tile
-      const int pairs = (a.mtiles + 1) / 2 * a.ntiles;
-      const int clusters = std::max(1, std::min(pairs, ds->ctx->sm_count / 2));
-      kern<<<2 * clusters, kThreads, smem, ds->ctx->stream>>>(st->A[0], st->A[1], st->A[2], mBh,
-                                                              st->J2[0], st->J2[1], st->J2[2],
-                                                              a);
       ISING_CUDA(ds->ctx, cudaGetLastError());
       return ISING_OK;
     }
@@ -2955,7 +2902,7 @@ int tc_bn(const ising_ds* ds) { return static_cast<const TcState*>(ds->tc)->BN; 
 
 int tc_tile_pair(const ising_ds* ds) {
   auto st = static_cast<const TcState*>(ds->tc);
-  return st->pair ? (st->split ? 2 : 1) : 0;
+  return st->pair ? 2 : 0;
 }
 
 // Restart-tile widths the streaming form can take for this session (tiles at
@@ -2966,15 +2913,11 @@ int tc_bn_candidates(const ising_ds* ds, int* out) {
   int k = 0;
   for (int bn : {64, 128, 224, 256})
     if (bn == 64 || bn / 2 < ds->B) out[k++] = bn;
-  // the same wide tiles over clusters of two CTAs sharing spin tiles
-  // (kTcPair: a flag on the width; with kTcSplit their MMAs run as one),
-  // when there are two row tiles to pair
+  // the same wide tiles over clusters of two CTAs (kTcPair: a flag on the
+  // width), when there are two row tiles to pair
   if (!ds->relaxed() && ds->n > kBM)
     for (int bn : {224, 256})
-      if (bn / 2 < ds->B) {
-        out[k++] = bn | kTcPair;
-        out[k++] = bn | kTcPair | kTcSplit;
-      }
+      if (bn / 2 < ds->B) out[k++] = bn | kTcPair;
   return k;
 }
 
@@ -2984,13 +2927,11 @@ int tc_bn_candidates(const ising_ds* ds, int* out) {
 int tc_set_bn(ising_ds* ds, int code) {
   auto st = static_cast<TcState*>(ds->tc);
   if (st->resident) return fail(ds->ctx, ISING_EINVAL, "tile width of a resident form");
-  const int bn = code & ~(kTcPair | kTcSplit);
+  const int bn = code & ~kTcPair;
   const bool pair = (code & kTcPair) != 0 && bn >= 192 && !ds->relaxed();
-  const bool split = pair && (code & kTcSplit) != 0;
-  if (st->BN == bn && st->pair == pair && st->split == split) return ISING_OK;
+  if (st->BN == bn && st->pair == pair) return ISING_OK;
   st->BN = bn;
   st->pair = pair;
-  st->split = split;
   st->maps_ready = false;
   st->trace.release();
   const int tiles = ceil_div_i(ds->n, kBM) * ceil_div_i(ds->B, bn);

@@ -145,19 +145,6 @@ __device__ __forceinline__ void tma_load_2d_to_pair(void* dst, const CUtensorMap
       : "memory");
 }
 
-// 2D tiled TMA load multicast to the CTAs of `mask` in the cluster: the box
-// lands at the offset of `dst` in the shared memory of each, and each one's
-// mbarrier at the offset of `bar` receives the bytes it got.
-__device__ __forceinline__ void tma_load_2d_mc(void* dst, const CUtensorMap* map, uint64_t* bar,
-                                               int c0, int c1, uint16_t mask, uint64_t policy) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      ".multicast::cluster.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5, %6;" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "h"(mask),
-      "l"(policy)
-      : "memory");
-}
-
 // Rank of this CTA in its cluster, the cluster's index and the number of
 // clusters (1D grids).
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -330,16 +317,6 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile(
       "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
           smem_u32(bar))
-      : "memory");
-}
-
-// The same, arriving on the mbarrier at the offset of `bar` in each CTA of
-// `mask` in the cluster.
-__device__ __forceinline__ void mma_commit_mc(uint64_t* bar, uint16_t mask) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
-      " [%0], %1;" ::"r"(smem_u32(bar)),
-      "h"(mask)
       : "memory");
 }
 
