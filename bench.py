@@ -187,7 +187,8 @@ def launches_per_solve(T: int, rounds: int, path: int, resident: bool, rowsum: b
     field 3), session set-up (fills 2, init 1, operand 1, plus the row-sum
     bound when the tensor-core path accumulates integer energies: `rowsum`,
     plus the per-row scales of row-scaled operands: `rowscale`), the steps
-    (one launch when resident; on the streaming tensor-core path one launch
+    (one launch when resident, after three that lay out the couplings on the
+    sparse path; on the streaming tensor-core path one launch
     per step, each also tracking its predecessor, plus one tracking launch
     for the last step; else step + track per step, plus the copy of improved
     bit-packed spins on the sparse path, which the next step's tracking
@@ -195,7 +196,7 @@ def launches_per_solve(T: int, rounds: int, path: int, resident: bool, rowsum: b
     + track (+ copy) + argmin), reconstruction (1), full-instance energy (2)."""
     per_step = 3 if path == 2 else 2
     if resident:
-        steps = 1
+        steps = 4 if path == 2 else 1
     elif path == 1:
         steps = T + 1
     else:
@@ -627,6 +628,8 @@ def roofline(ctx, inst, dinst, name, B, kw, steps, pk, sessions=1):
         roof = {"bound": "hbm", "achieved": alg / (avg_ms / 1e3) / 1e9, "peak": pk["hbm_gbs"],
                 "unit": "GB/s", "peak_note": "measured copy bandwidth"}
         kname, ksrc = "sparse_step_kernel", "paper_2312_05837_gb300/csrc/ds_sparse.cu"
+        if st["resident"]:  # (the state then stays in shared memory: alg is what a step per launch moves)
+            kname, ksrc = "sparse_res_kernel", "paper_2312_05837_gb300/csrc/ds_sparse_res.cu"
     elif path == 1:  # tensor cores: 2 N^2 B flop per step
         alg = 2.0 * n * n * B
         fp8 = st["precision"] == 4
@@ -809,7 +812,7 @@ def main():
             "gpu_launches": launches_per_solve(
                 T, rounds, path, bool(last["resident"]), path == 1 and bool(inst.integer),
                 path == 1 and not inst.integer and prec in (2, 4),
-                path == 2 and n_red > 4096) * a.steps,
+                path == 2 and n_red > 4096 and not last["resident"]) * a.steps,
             "roofline": roof, "clocks": clk,
             "best_energy": float(last["best_energy"].item())}
     if name.startswith("table2"):

@@ -122,15 +122,16 @@ typedef struct ising_ds_params {
 } ising_ds_params;
 
 /* params.flags: time every step-kernel launch with CUDA events on the
- * context's stream and report the sum in ising_ds_stats.kernel_ms (for the
- * resident tensor-core form, one launch runs many steps: kernel_ms / kernel_launches
- * is then the time per step). */
+ * context's stream and report the sum in ising_ds_stats.kernel_ms (a resident
+ * form runs many steps per launch: kernel_ms / kernel_launches is then the
+ * time per step). */
 #define ISING_DS_PROFILE 1
 /* params.flags: keep the state in device memory between steps (one launch
  * per step) even when a resident form would fit. The resident form of the
  * sparse path runs a whole run of steps in one launch with the state of each
  * block's restarts in shared memory (instances whose spins, state and one to
- * eight restarts fit there). The tensor-core path's resident forms keep theta, m and v in tensor memory across a whole run in
+ * eight restarts fit there). The tensor-core path's resident forms keep theta,
+ * m and v in tensor memory across a whole run in
  * one launch: for n <= 128 the small form (every CTA holds all of J and the
  * spins of its block of 16 to 128 restarts in shared memory, no grid-wide
  * barrier), for larger n the grid-wide form (one cooperative launch), used
@@ -177,9 +178,10 @@ typedef struct ising_ds_stats {
   double device_ms;         /* device time of the steps (CUDA events) */
   double kernel_ms;         /* step kernels only (with ISING_DS_PROFILE) */
   int64_t kernel_launches;  /* step-kernel launches timed in kernel_ms */
-  int32_t resident;         /* tensor-core path kept the state in tensor memory: 1 in the
-                               grid-wide form, 2 in the small form (n <= 128, each CTA holds
-                               all of J and its restarts' spins on chip); 0 otherwise */
+  int32_t resident;         /* form that runs all steps of a run in one launch: 1 the tensor
+                               cores' grid-wide form, 2 their small form (n <= 128, each CTA
+                               holds all of J and its restarts' spins on chip), 3 the sparse
+                               path's (a block's restarts in shared memory); 0 a launch per step */
   int32_t operand_planes;   /* tensor-core path: operand planes of J per product (1 or 2;
                                the tensor cores execute that many products), else 1 */
   int32_t tile_restarts;    /* tensor-core streaming form: restarts per tile, else 0 */

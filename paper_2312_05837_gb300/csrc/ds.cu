@@ -1401,7 +1401,7 @@ extern "C" int ising_ds_result(ising_ds* ds, int8_t* best_spins, double* best_en
     stats->device_ms = ds->device_ms;
     stats->kernel_ms = ds->kernel_ms;
     stats->kernel_launches = ds->kernel_launches;
-    stats->resident = ds->path == ISING_PATH_TC ? tc_resident_form(ds) : 0;
+    stats->resident = ds->path == ISING_PATH_TC ? tc_resident_form(ds) : (ds->sres ? 3 : 0);
     stats->operand_planes = ds->path == ISING_PATH_TC ? ds->planes : 1;
     const bool streaming = ds->path == ISING_PATH_TC && tc_resident_form(ds) == 0;
     stats->tile_restarts = streaming ? tc_bn(ds) : 0;

@@ -612,9 +612,8 @@ int sr_launch_pack(ising_ds* ds, const SparseRes* R, const SrArgs& a) {
 }  // namespace
 
 // Whether the session runs this form, and its operands. It does when the
-// state of RB restarts fits a CTA's shared memory (n RB up to about 18000,
-// 14000 with 16-bit spins),
-// with RB the least of 1, 2, 4, 8 that gives every SM at most one CTA, or 8
+// state of RB restarts fits a CTA's shared memory (n RB up to about 16300,
+// 14300 with 16-bit spins), with RB the least of 1, 2, 4, 8 that gives every SM at most one CTA, or 8
 // (several waves of CTAs then): the launch-per-step form costs at least two
 // launches and an L2 round trip per coupling however small the instance.
 int sparse_res_setup(ising_ds* ds) {
