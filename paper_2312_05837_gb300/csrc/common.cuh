@@ -166,6 +166,7 @@ struct DevInstance {
   double j_absmax = 0.0;    // max |J|
   int64_t j_nonzeros = 0;   // dense: non-zero J values, and the sum of their
   int64_t j_expsum = 0;     // binary exponents (floor log2 |J|)
+  int row_max = 0;          // CSR: entries of the longest row
   bool h_dyadic = true;     // every h * 2^h_shift is an integer of |.| < 2^30
   int h_shift = 0;
   double h_absmax = 0.0;

@@ -6,7 +6,7 @@
 //            in integers whatever the order, rounded once at the end;
 //   planes   dense J and many vectors: the same integers as digits in FP16
 //            planes, their sums on the tensor cores, exact as well;
-//   packed   CSR, 8 or more vectors: a lane per vector, spins as bits;
+//   packed   CSR without long rows, many vectors: a lane per vector, spins as bits;
 //   general  a warp per row and vector, int64 or FP64: few CSR vectors, dense J
 //            whose values spread too widely for one scale, the call without
 //            allocation, and spins that are not +-1.
@@ -484,6 +484,63 @@ __global__ void __launch_bounds__(256) pack_sites_kernel(const int8_t* __restric
   }
 }
 
+constexpr int kPackedRow = 128;  // the longest row of an instance in this form
+constexpr int kPackedLevels = 6;  // its 32 groups of four entries in the counter
+
+// (J s)_i of the lane's vector over the row's entries [e0, e1). Integers in
+// order; FP64 pairwise, four entries by a tree and the groups of four by a
+// binary counter (level l holds the sum of 2^l groups), so that no entry passes
+// through more additions than in the general form's lanes and tree: in order,
+// the error of rows of 64 entries was 1.6 times that form's.
+template <bool INT, typename Acc = typename std::conditional<INT, long long, double>::type>
+__device__ __forceinline__ Acc packed_row(const RowsView<int32_t>& in, const uint32_t* __restrict__ bits,
+                                          int64_t words, int e0, int e1, int lane) {
+  auto term = [&](int e) {
+    const uint32_t w = bits[(int64_t)in.indices[e] * words];
+    Acc x;
+    if constexpr (INT) x = (Acc)load_as_int(in.J, in.j_dtype, e);
+    else x = (Acc)load_as_double(in.J, in.j_dtype, e);
+    return (w >> lane) & 1u ? x : -x;
+  };
+  if constexpr (INT) {
+    Acc dot = 0;
+#pragma unroll 4
+    for (int e = e0; e < e1; ++e) dot += term(e);
+    return dot;
+  } else {
+    Acc level[kPackedLevels];
+#pragma unroll
+    for (int l = 0; l < kPackedLevels; ++l) level[l] = 0;
+#pragma unroll 1
+    for (int e = e0; e < e1; e += 4) {
+      Acc x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const Acc y = term(e + u < e1 ? e + u : e0);
+        x[u] = e + u < e1 ? y : (Acc)0;
+      }
+      Acc sum = (x[0] + x[1]) + (x[2] + x[3]);
+      const int g = (e - e0) >> 2;  // (uniform over the warp)
+      bool carry = true;
+#pragma unroll
+      for (int l = 0; l < kPackedLevels; ++l)
+        if (carry) {
+          if (l + 1 < kPackedLevels && ((g >> l) & 1)) {
+            sum += level[l];
+            level[l] = 0;
+          } else {
+            level[l] += sum;  // (empty, or the last level)
+            carry = false;
+          }
+        }
+    }
+    Acc dot = level[0];
+#pragma unroll
+    for (int l = 1; l < kPackedLevels; ++l) dot += level[l];
+    return dot;
+  }
+}
+
 // Block: kRowsPerBlock rows (warp w takes every 8th), 32 vectors (blockIdx.y);
 // partials as the general form's, [vector][block].
 template <bool INT>
@@ -498,16 +555,7 @@ __global__ void __launch_bounds__(256) energy_packed_kernel(RowsView<int32_t> in
   Acc q = 0, hs = 0;
   const int64_t r0 = (int64_t)blockIdx.x * kRowsPerBlock;
   for (int64_t i = r0 + warp; i < r0 + kRowsPerBlock && i < in.n; i += 8) {
-    const int e1 = in.rowptr[i + 1];
-    Acc dot = 0;
-#pragma unroll 4
-    for (int e = in.rowptr[i]; e < e1; ++e) {
-      const uint32_t w = bits[(int64_t)in.indices[e] * words + blockIdx.y];
-      Acc x;
-      if (INT) x = (Acc)load_as_int(in.J, in.j_dtype, e);
-      else x = (Acc)load_as_double(in.J, in.j_dtype, e);
-      dot += (w >> lane) & 1u ? x : -x;
-    }
+    const Acc dot = packed_row<INT>(in, bits + blockIdx.y, words, in.rowptr[i], in.rowptr[i + 1], lane);
     const bool up = (bits[i * words + blockIdx.y] >> lane) & 1u;
     q += up ? dot : -dot;
     if (in.h) {
@@ -671,9 +719,21 @@ int energy_packed(ising_ctx* ctx, const DevInstance& inst, bool exact, const int
 // n = 4096 FP32: 256 vectors 23.5 ms in the general form, 2.5 in the fixed, 0.2
 // in planes; one vector of n = 1000: 166 -> 6.4 us;
 // but small integer ones, whose general form takes fewer launches: n = 121, 51
-// vectors 99 against 109 us per call), the packed form for 8 or more vectors of
-// a CSR instance (below that its lanes are as idle as the general form's), the
-// general form otherwise and whenever a spin is not +-1.
+// vectors 99 against 109 us per call), the packed form for CSR instances where
+// packed_pays, the general form otherwise and whenever a spin is not +-1.
+//
+// The packed form: a launch and a host read more (about 25 us a call), and a
+// warp walks a row alone, but a row of 32 vectors costs one warp instead of 32
+// (0.15 ns each with integers, 0.55 in FP64). us per call, general / packed, n
+// 20000: int8 of degree 4 and 8, 16, 32 vectors 187 / 188, 213 / 185, 262 / 185;
+// of degree 128, 8 and 256 vectors 465 / 525, 1301 / 926; FP64 of degree 64, 8
+// and 32 vectors 407 / 609, 737 / 612. n = 1000 of degree 8: int8, 32 and 256
+// vectors 173 / 196, 210 / 201; FP64 187 / 197, 310 / 203.
+bool packed_pays(const DevInstance& I, bool exact, int64_t count) {
+  const int64_t row = std::min<int64_t>(kPackedRow, exact ? count : 2 * count);
+  return count >= 8 && I.row_max <= row && (double)I.n * (double)count >= (exact ? 131072.0 : 65536.0);
+}
+
 int energy_device(ising_ctx* ctx, const DevInstance& inst, const int8_t* spins, int64_t count,
                   double* E, int64_t* Q, int64_t* H) {
   if (count <= 0) return ISING_OK;
@@ -685,7 +745,7 @@ int energy_device(ising_ctx* ctx, const DevInstance& inst, const int8_t* spins, 
     const double terms = (double)inst.n * (double)inst.n * (double)count;
     if (!(exact && terms < 2097152.0) && fixed_scale(inst, &shift))
       ISING_TRY(energy_fixed(ctx, inst, exact, shift, spins, count, E, Q, H, &ok));
-  } else if (count >= 8) {
+  } else if (packed_pays(inst, exact, count)) {
     ISING_TRY(energy_packed(ctx, inst, exact, spins, count, E, Q, H, &ok));
   }
   return ok ? ISING_OK : energy_general(ctx, inst, exact, spins, count, E, Q, H);

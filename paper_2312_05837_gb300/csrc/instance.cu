@@ -18,6 +18,7 @@ struct ValFlags {
   unsigned long long h_absmax;
   unsigned long long j_nonzeros;  // dense: non-zero J values, and the sum of
   long long j_expsum;             // their binary exponents (floor log2 |J|)
+  int row_max;                    // CSR: entries of the longest row
 };
 
 // Facts gathered per thread and merged once per warp (a same-address atomic
@@ -161,14 +162,18 @@ __global__ void __launch_bounds__(256) check_dense(const T* __restrict__ J, int6
 
 __global__ void check_indptr(const int64_t* indptr, int64_t n, int64_t nnz, int32_t* rowptr,
                              ValFlags* f) {
+  int64_t longest = 0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= n;
        i += (int64_t)gridDim.x * blockDim.x) {
     int64_t a = indptr[i];
     if (i == 0 && a != 0) atomicOr(&f->bad, 8u);
     if (i == n && a != nnz) atomicOr(&f->bad, 8u);
     if (i < n && indptr[i + 1] < a) atomicOr(&f->bad, 8u);
+    if (i < n && indptr[i + 1] - a > longest) longest = indptr[i + 1] - a;
     rowptr[i] = (int32_t)a;
   }
+  const int m = __reduce_max_sync(0xffffffffu, (int)min(longest, (int64_t)INT32_MAX));
+  if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(&f->row_max, m);
 }
 
 // CSR rows: columns in range, strictly increasing, no diagonal; each (i,j,v)
@@ -351,6 +356,7 @@ int upload_instance(ising_ctx* ctx, const ising_instance* in, DevInstance* out, 
   out->j_absmax = bits_to_double(fh.j_absmax);
   out->j_nonzeros = (int64_t)fh.j_nonzeros;
   out->j_expsum = fh.j_expsum;
+  out->row_max = fh.row_max;
   out->h_absmax = in->h ? bits_to_double(fh.h_absmax) : 0.0;
   out->h_dyadic = true;
   out->h_shift = 0;
