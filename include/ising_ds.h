@@ -221,9 +221,10 @@ int ising_selftest_waits(ising_ctx* ctx, int64_t limit_cycles, int32_t* gave_up)
  * `mem`). Writes E_out[count] (float64) and, if Q_out / H_out are not NULL
  * and the instance is integer, the exact parts Q = s^T J s and H = h^T s
  * (int64, E = cQ Q + cH H). Integer couplings accumulate in integers and
- * are exact; other couplings accumulate in FP64, or for spins of +-1 in fixed
- * point of more bits (many vectors of a dense instance: as exact FP16 digits
- * of the couplings on the tensor cores). Outputs are in memory `mem`. */
+ * are exact; other couplings accumulate in FP64, or, for spins of +-1 and a
+ * dense instance, as integers of up to 58 bits of one scale for the matrix whose
+ * roundings together stay below 2^-53 sum |J_ij| (many vectors: as exact FP16
+ * digits of those integers on the tensor cores). Outputs are in memory `mem`. */
 int ising_energy(ising_ctx* ctx, const ising_instance* inst, const int8_t* spins,
                  int64_t count, double* E_out, int64_t* Q_out, int64_t* H_out, int mem);
 

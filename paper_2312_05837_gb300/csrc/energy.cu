@@ -177,13 +177,14 @@ __device__ __forceinline__ long long to_fixed(T x, int shift, double dscale) {
   }
 }
 
-// Block: rows 4 blockIdx.x .. + 3, vectors V blockIdx.y .. ; warp w takes every
-// 8th group of 32 VEC columns, lane l of it VEC consecutive ones (VEC = 4 needs
-// n % 4 == 0, so that every row starts on a vector boundary).
+// Block: rows 4 blockIdx.x .. + 3, vectors V blockIdx.y .., the blockIdx.z-th
+// `span` columns (a multiple of 1024); warp w takes every 8th group of 32 VEC
+// columns, lane l of it VEC consecutive ones (VEC = 4 needs n % 4 == 0, so that
+// every row starts on a vector boundary).
 // limbs[v][3] receives the limbs of s^T I s.
 template <typename T, int VEC, int V>
 __global__ void __launch_bounds__(256) energy_fixed_kernel(
-    int64_t n, const T* __restrict__ J, int shift, double dscale,
+    int64_t n, int64_t span, const T* __restrict__ J, int shift, double dscale,
     const uint32_t* __restrict__ bits, int64_t words, int64_t count,
     unsigned long long* __restrict__ limbs) {
   extern __shared__ uint32_t sbits[];  // [V][words]
@@ -202,9 +203,14 @@ __global__ void __launch_bounds__(256) energy_fixed_kernel(
 #pragma unroll
     for (int v = 0; v < V; ++v) acc[r][v] = 0;
   }
-  const int64_t groups = (n + 32 * VEC - 1) / (32 * VEC);
+  int64_t g = warp, groups = (n + 32 * VEC - 1) / (32 * VEC);
+  if constexpr (std::is_same<T, double>::value) {  // (the only type whose columns are split)
+    const int64_t per = span / (32 * VEC);
+    g += blockIdx.z * per;
+    groups = min(groups, (blockIdx.z + 1) * per);
+  }
 #pragma unroll 2
-  for (int64_t g = warp; g < groups; g += 8) {
+  for (; g < groups; g += 8) {
     const int64_t j = (g * 32 + lane) * VEC;
     T x[kFixRows][VEC];
 #pragma unroll
@@ -307,58 +313,75 @@ __global__ void __launch_bounds__(256) energy_fixed_finish(
   }
 }
 
-// The binary scale of the fixed form: 0 for integer couplings; else
-// every J_ij becomes rint(J_ij 2^*shift) with b bits, b the most for which no
-// lane's sums overflow. Each rounding is off by at most 2^-(b + 1) 2^E
-// (|J| < 2^E), all of them together by no more than 16 2^-53 sum |J_ij|, which
-// is below the bound of an FP64 sum of that many terms in any order (at least
-// log2(n^2) 2^-53 sum |J_ij|, 16 at n = 256; a smaller sum has more bits to
-// spare), or else the form is not used. sum |J_ij| is at least the count of
-// non-zeros times their geometric mean, which the mean exponent bounds below.
+// The binary scale of the integer forms: 0 for integer couplings; else every
+// J_ij becomes rint(J_ij 2^*shift) with b bits (|J| < 2^E, largest b bits), and
+// the form is used only where all those roundings together stay below 2^-53
+// sum |J_ij|, what rounding each coupling once to FP64 may cost. Each is off by
+// at most 2^-(b + 1) 2^E, and sum |J_ij| is at least the count of non-zeros times
+// their geometric mean, which the mean exponent bounds below: so FP64 couplings
+// need a mean exponent of E - b + 52. FP32 couplings have 24 bits: those above
+// 2^(E - b + 24) are exact, and where the mean exponent is at least E - b + 48 at
+// most 4 / 15 of the others' number can lie below that, whose roundings add up to
+// less than 2^-54 sum |J_ij|.
 bool scale_for(const DevInstance& I, int b, int* shift) {
   int ex = 0;
   std::frexp(I.j_absmax, &ex);  // |J| < 2^ex
-  if ((double)I.j_expsum < (double)(ex - b + 48) * (double)I.j_nonzeros) return false;
+  const int need = I.j_dtype == ISING_F64 ? 52 : 48;
+  if ((double)I.j_expsum < (double)(ex - b + need) * (double)I.j_nonzeros) return false;
   *shift = b - ex;
   return *shift >= -120 && *shift <= 120;  // a float power of two; no result underflows
 }
+
+// Columns of one block of the fixed form when `splits` blocks share a row: whole
+// groups of every warp and lane.
+int64_t split_columns(int64_t n, int splits) { return ((n + splits - 1) / splits + 1023) / 1024 * 1024; }
 
 // Integer couplings that the integer forms add as they are (scale 0): whatever
 // the fields, whose sum of a non-dyadic h stays in FP64.
 bool whole_couplings(const DevInstance& I) { return I.j_integer && I.j_absmax <= 2147483648.0; }
 
-bool fixed_scale(const DevInstance& I, int* shift) {
+// b for the fixed form: the most for which no lane's sums overflow, with the
+// columns dealt to *splits blocks where FP64 couplings need the bits (n = 8192
+// Gaussian: one lane's 32 terms leave 56 bits, two blocks' 16 leave 57).
+bool fixed_scale(const DevInstance& I, int* shift, int* splits) {
   *shift = 0;
+  *splits = 1;
   if (whole_couplings(I) || I.j_nonzeros == 0) return true;
-  const int64_t lane_terms = 4 * ((I.n + 1023) / 1024) + 4;
-  int lg = 0;
-  while (((int64_t)1 << lg) < lane_terms) ++lg;
-  return scale_for(I, std::min(58, 61 - lg), shift);
+  for (;; *splits *= 2) {
+    const int64_t lane_terms = 4 * ((split_columns(I.n, *splits) + 1023) / 1024);
+    int lg = 0;
+    while (((int64_t)1 << lg) < lane_terms) ++lg;
+    const int b = std::min(58, 61 - lg);
+    if (scale_for(I, b, shift)) return true;
+    if (b == 58 || I.j_dtype != ISING_F64) return false;
+  }
 }
 
 template <typename T, int VEC>
-int fixed_launch(ising_ctx* ctx, const DevInstance& I, int shift, const uint32_t* bits,
+int fixed_launch(ising_ctx* ctx, const DevInstance& I, int shift, int splits, const uint32_t* bits,
                  int64_t words, int64_t count, unsigned long long* limbs) {
   const double dsc = std::ldexp(1.0, shift);
   const int V = count == 1 ? 1 : kFixVectors;
-  const dim3 grid((unsigned)((I.n + kFixRows - 1) / kFixRows), (unsigned)((count + V - 1) / V));
+  const int64_t span = split_columns(I.n, splits);
+  const dim3 grid((unsigned)((I.n + kFixRows - 1) / kFixRows), (unsigned)((count + V - 1) / V),
+                  (unsigned)((I.n + span - 1) / span));
   const size_t smem = (size_t)V * words * 4;
   if (V == 1)
     energy_fixed_kernel<T, VEC, 1><<<grid, 256, smem, ctx->stream>>>(
-        I.n, I.J.as<T>(), shift, dsc, bits, words, count, limbs);
+        I.n, span, I.J.as<T>(), shift, dsc, bits, words, count, limbs);
   else
     energy_fixed_kernel<T, VEC, kFixVectors><<<grid, 256, smem, ctx->stream>>>(
-        I.n, I.J.as<T>(), shift, dsc, bits, words, count, limbs);
+        I.n, span, I.J.as<T>(), shift, dsc, bits, words, count, limbs);
   ISING_CUDA(ctx, cudaGetLastError());
   return ISING_OK;
 }
 
 template <typename T>
-int fixed_launch_t(ising_ctx* ctx, const DevInstance& I, int shift, const uint32_t* bits,
+int fixed_launch_t(ising_ctx* ctx, const DevInstance& I, int shift, int splits, const uint32_t* bits,
                    int64_t words, int64_t count, unsigned long long* limbs) {
   // rows of a multiple of four values start on a vector boundary
-  return I.n % 4 == 0 ? fixed_launch<T, 4>(ctx, I, shift, bits, words, count, limbs)
-                      : fixed_launch<T, 1>(ctx, I, shift, bits, words, count, limbs);
+  return I.n % 4 == 0 ? fixed_launch<T, 4>(ctx, I, shift, splits, bits, words, count, limbs)
+                      : fixed_launch<T, 1>(ctx, I, shift, splits, bits, words, count, limbs);
 }
 
 // --------------------------------------------------------------- planes form
@@ -440,7 +463,7 @@ bool plane_scale(const DevInstance& I, int* w, int* planes, int* shift) {
     *planes = (bits + 1 + *w - 1) / *w;
     return true;
   }
-  for (*planes = 4; *planes <= 7; ++*planes)
+  for (*planes = 5; *planes <= 7; ++*planes)
     if (scale_for(I, std::min(58, *w * *planes - 2), shift)) return true;
   return false;
 }
@@ -644,7 +667,7 @@ int plane_limbs(ising_ctx* ctx, const DevInstance& inst, int w, int planes, int 
   return ISING_OK;
 }
 
-int energy_fixed(ising_ctx* ctx, const DevInstance& inst, bool exact, int shift,
+int energy_fixed(ising_ctx* ctx, const DevInstance& inst, bool exact, int shift, int splits,
                  const int8_t* spins, int64_t count, double* E, int64_t* Q, int64_t* H, bool* ok) {
   const int64_t n = inst.n, words = (n + 31) / 32;
   DevMem work;  // limbs [count][3], the flag (8 bytes), bits [count][words]
@@ -664,10 +687,10 @@ int energy_fixed(ising_ctx* ctx, const DevInstance& inst, bool exact, int shift,
   if (rc == ISING_OK) shift = pshift;
   else if (rc != ISING_ENOMEM) return rc;
   else switch (inst.j_dtype) {
-    case ISING_F64: ISING_TRY(fixed_launch_t<double>(ctx, inst, shift, bw, words, count, L)); break;
-    case ISING_F32: ISING_TRY(fixed_launch_t<float>(ctx, inst, shift, bw, words, count, L)); break;
-    case ISING_I8: ISING_TRY(fixed_launch_t<int8_t>(ctx, inst, shift, bw, words, count, L)); break;
-    default: ISING_TRY(fixed_launch_t<int32_t>(ctx, inst, shift, bw, words, count, L)); break;
+    case ISING_F64: ISING_TRY(fixed_launch_t<double>(ctx, inst, shift, splits, bw, words, count, L)); break;
+    case ISING_F32: ISING_TRY(fixed_launch_t<float>(ctx, inst, shift, splits, bw, words, count, L)); break;
+    case ISING_I8: ISING_TRY(fixed_launch_t<int8_t>(ctx, inst, shift, splits, bw, words, count, L)); break;
+    default: ISING_TRY(fixed_launch_t<int32_t>(ctx, inst, shift, splits, bw, words, count, L)); break;
   }
   const void* h = inst.has_h ? inst.h.p : nullptr;
   const double unscale = std::ldexp(1.0, -shift);
@@ -740,11 +763,11 @@ int energy_device(ising_ctx* ctx, const DevInstance& inst, const int8_t* spins, 
   const bool exact = inst.j_integer && inst.j_absmax < 2147483648.0 && inst.h_dyadic;
   if (count > 65535) return fail(ctx, ISING_EINVAL, "energy: count > 65535 per call");
   bool ok = false;
-  int shift = 0;
+  int shift = 0, splits = 1;
   if (inst.layout == ISING_LAYOUT_DENSE) {
     const double terms = (double)inst.n * (double)inst.n * (double)count;
-    if (!(exact && terms < 2097152.0) && fixed_scale(inst, &shift))
-      ISING_TRY(energy_fixed(ctx, inst, exact, shift, spins, count, E, Q, H, &ok));
+    if (!(exact && terms < 2097152.0) && fixed_scale(inst, &shift, &splits))
+      ISING_TRY(energy_fixed(ctx, inst, exact, shift, splits, spins, count, E, Q, H, &ok));
   } else if (packed_pays(inst, exact, count)) {
     ISING_TRY(energy_packed(ctx, inst, exact, spins, count, E, Q, H, &ok));
   }
