@@ -341,10 +341,12 @@ int plain_setup(ising_ds* ds);
 int plain_step(ising_ds* ds, int mode, float* Gout);
 int sparse_setup(ising_ds* ds);
 int sparse_step(ising_ds* ds, int mode, float* Gout);
+constexpr int64_t kSparseResMaxSpins = 16600;  // 14 bytes each in 227 KB of shared memory
 int sparse_res_setup(ising_ds* ds);  // chooses the resident form (ds->sres) where it applies
 int sparse_res_run(ising_ds* ds, int64_t steps);  // queues `steps` steps, advances ds->t
 void sparse_res_release(ising_ds* ds);
 int tc_setup(ising_ds* ds);
+int64_t tc_pitch(int64_t n, bool fp8);  // row pitch of its operands and state
 int tc_step(ising_ds* ds, int mode, float* Gout);
 int tc_error(ising_ds* ds);  // ISING_ETIMEOUT if a bounded wait gave up
 bool tc_is_resident(ising_ds* ds);            // tensor memory keeps the state between steps

@@ -621,7 +621,7 @@ int sparse_res_setup(ising_ds* ds) {
   if ((ds->p.flags & ISING_DS_STREAMING) || ds->relaxed()) return ISING_OK;
   const DevInstance& I = ds->inst;
   const int64_t n = ds->n, nnz = I.nnz;
-  if (n > 20000 || nnz > (1 << 24)) return ISING_OK;
+  if (n > kSparseResMaxSpins || nnz > (1 << 24)) return ISING_OK;
   const bool v8 = ds->sp_int8;
   if (ds->int_energy) {
     // energies and fields are added in 32 bits

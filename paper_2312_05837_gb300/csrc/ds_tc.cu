@@ -2419,6 +2419,17 @@ static size_t gsync_bytes(const ising_ds* ds, const TcState* st) {
   return (size_t)(1 + st->gr * ceil_div_i(ds->B, st->gr * st->gn)) * 128;
 }
 
+// Row pitch (elements) of the operands and the state: 16-byte rows, or rows of
+// whole 128-byte lines where that adds at most 1/16: a TMA box then copies at 83
+// to 93 bytes per cycle and SM instead of 49 to 73 (resident form, 1999 spins x
+// 1024 restarts x 2000 steps: 23.8 -> 22.7 ms; 1000 spins in two planes 13.69 ->
+// 13.55). Smaller instances are not bound by copies and keep the smaller state.
+int64_t tc_pitch(int64_t n, bool fp8) {
+  const int64_t ld = fp8 ? (n + 15) / 16 * 16 : (n + 7) / 8 * 8;
+  const int64_t line = fp8 ? (n + 127) / 128 * 128 : (n + 63) / 64 * 64;
+  return 16 * (line - ld) <= ld ? line : ld;
+}
+
 int tc_setup(ising_ds* ds) {
   ising_ctx* ctx = ds->ctx;
   const DevInstance& I = ds->inst;
@@ -2437,14 +2448,7 @@ int tc_setup(ising_ds* ds) {
   // AUTO: E4M3 when it holds J exactly, else the exact BF16 form
   if (ds->prec == ISING_PREC_AUTO) ds->prec = exact16 ? ISING_PREC_FP8 : ISING_PREC_TC;
   st->fp8 = ds->prec == ISING_PREC_FP8;
-  ds->ld = st->fp8 ? (ds->n + 15) / 16 * 16 : (ds->n + 7) / 8 * 8;
-  // Operand rows of whole 128-byte lines where that adds at most 1/16: a TMA
-  // box then copies at 83 to 93 bytes per cycle and SM instead of 49 to 73
-  // (resident form, 1999 spins x 1024 restarts x 2000 steps: 23.8 -> 22.7 ms;
-  // 1000 spins in two planes 13.69 -> 13.55). Smaller instances are not bound
-  // by copies and keep the smaller state.
-  const int64_t line = st->fp8 ? (ds->n + 127) / 128 * 128 : (ds->n + 63) / 64 * 64;
-  if (16 * (line - ds->ld) <= ds->ld) ds->ld = line;
+  ds->ld = tc_pitch(ds->n, st->fp8);
   ds->Bp = ds->B;
   ds->spin_kind = st->fp8 ? kSpinE4M3 : kSpinBF16;
   ds->mtiles = 4 * ceil_div_i(ds->n, kBM);  // one energy-partial row per epilogue lane quarter

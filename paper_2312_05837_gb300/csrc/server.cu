@@ -82,9 +82,9 @@ enum Phase { kQueued = 0, kSettingUp, kReady, kFinishing, kDone };
 
 constexpr int kPackStreams = 4;  // streams the server's packs take in turn
 
-// Device bytes a request holds while admitted (instance copy, pruning work,
-// operands, state, spins, partials, bests), estimated from its shape.
-size_t estimate_footprint(const ising_instance* in, const ising_ds_params* p) {
+// Device bytes of a request's instance, operands, state and bests: one that
+// takes more than the budget is refused.
+size_t core_footprint(const ising_instance* in, const ising_ds_params* p) {
   const double n = (double)in->n, B = (double)p->restarts;
   const double ld = n + 16.0;
   const double jsz = (double)dtype_size(in->j_dtype);
@@ -102,6 +102,53 @@ size_t estimate_footprint(const ising_instance* in, const ising_ds_params* p) {
   bytes += 2.0 * B * (4.0 * (n / 128.0 + 1.0)) * 20.0;  // energy partials
   bytes += 4.0 * 1024.0 * 1024.0;               // small buffers
   return (size_t)bytes;
+}
+
+// Device bytes a request holds at most while admitted, from its shape: the
+// larger of pruning (the instance, its entries as a list, the reduced instance)
+// and the session (the instance, the reduced one and the session's copy of it,
+// operands, state, bests, and the final energies of up to 64 candidates).
+size_t footprint_bound(const ising_ctx* ctx, const ising_instance* in, const ising_ds_params* p) {
+  const int64_t ni = in->n;
+  const double n = (double)ni, B = (double)p->restarts;
+  const double jsz = (double)dtype_size(in->j_dtype);
+  const bool relaxed = (p->flags & ISING_DS_RELAXED) != 0;
+  double prune, session, rows;
+  double Bp = B;
+  if (in->layout == ISING_LAYOUT_DENSE) {
+    const double J = n * n * jsz;
+    prune = 2.0 * J + n * n * 12.0;
+    // AUTO may take either operand type
+    const bool plain = p->precision == ISING_PREC_FP32_PLAIN, fp8 = p->precision == ISING_PREC_FP8;
+    const double ld = plain ? n
+                      : fp8 ? (double)tc_pitch(ni, true)
+                            : (double)std::max(tc_pitch(ni, true), tc_pitch(ni, false));
+    const double spin = plain ? 4.0 : fp8 ? 1.0 : 2.0;
+    session = 3.0 * J + (plain || !fp8 ? 4.0 : 1.0) * n * ld +
+              B * ld * (12.0 + 3.0 * spin + (relaxed ? 2.0 * spin : 0.0));
+    // the digit planes of the candidates' energies (at most 7, for whole
+    // couplings 4), their spins and partial sums
+    const double cand = std::min(B, 64.0);
+    if (n <= 16384.0 && cand >= 16.0 && n * n * cand >= 268435456.0) {
+      const double planes = in->j_dtype == ISING_I8 || in->j_dtype == ISING_I32 ? 4.0 : 7.0;
+      session += planes * n * (n + 64.0) * 2.0 + cand * (n + 64.0) * 2.0 +
+                 (planes + 1.0) * (n / 32.0 + 4.0) * cand * 8.0;
+    }
+    rows = n / 32.0 + 4.0;  // of energy partials
+  } else {
+    const double nnz = (double)in->nnz, copy = nnz * (jsz + 4.0) + n * 20.0;
+    Bp = (double)((p->restarts + 127) / 128 * 128);
+    prune = 2.0 * copy + nnz * 8.0;
+    session = 3.0 * copy + nnz * 4.0 + Bp * n * (12.0 + 3.0 / 8.0 + (relaxed ? 8.0 : 0.0));
+    // slices of the resident form (they hold at most so many slots)
+    if (ni <= kSparseResMaxSpins && !relaxed && !(p->flags & ISING_DS_STREAMING))
+      session += (6.0 * nnz + 32768.0) * (in->j_dtype == ISING_I8 ? 4.0 : 8.0);
+    rows = std::min(n / 8.0 + 1.0, ctx->sm_count * 4.0 / (Bp / 128.0) + 1.0);
+  }
+  session += 2.0 * rows * Bp * 20.0 + B * (n + 16.0) + B * 96.0 + 64.0 * (n + 16.0) +
+             ((double)p->steps + 2.0) * 8.0 + n * 16.0;
+  // (pruning's per-spin arrays, the result's among them, and small buffers)
+  return (size_t)(std::max(prune, session) + n * 64.0 + 4.0 * 1024.0 * 1024.0);
 }
 
 }  // namespace
@@ -584,9 +631,11 @@ int submit_impl(ising_server* srv, const ising_instance* inst, const ising_ds_pa
     return fail(ctx, ISING_EINVAL, "CSR instance needs indptr and indices");
   if (p->restarts < 1 || p->steps < 0) return fail(ctx, ISING_EINVAL, "bad parameters");
   auto r = std::make_unique<Request>();
-  r->footprint = estimate_footprint(inst, p);
-  if (r->footprint > srv->cfg.budget_bytes)
-    return fail(ctx, ISING_EBUSY, "request footprint %zu exceeds the budget", r->footprint);
+  const size_t core = core_footprint(inst, p);
+  if (core > srv->cfg.budget_bytes)
+    return fail(ctx, ISING_EBUSY, "request footprint %zu exceeds the budget", core);
+  // (a request that fits the budget but for pruning or the final energies runs alone)
+  r->footprint = std::min<size_t>(footprint_bound(srv->parent, inst, p), srv->cfg.budget_bytes);
   const int64_t n = inst->n;
   const size_t jsz = dtype_size(inst->j_dtype);
   const size_t jcount = inst->layout == ISING_LAYOUT_DENSE ? (size_t)n * n : (size_t)inst->nnz;
