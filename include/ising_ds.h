@@ -214,6 +214,12 @@ int ising_version(void);
  * call returns ISING_ETIMEOUT, after which the context stays usable.
  * limit_cycles must lie in [1, 2^34]. */
 int ising_selftest_waits(ising_ctx* ctx, int64_t limit_cycles, int32_t* gave_up);
+/* Diagnostic of the behaviour at scratch limits (the paper has no
+ * counterpart): from now on a device allocation of this context above `bytes`
+ * fails as if memory had run out (0: no limit). Forms that need more scratch
+ * than the general ones then give way to them; what no form can do without
+ * makes the call return ISING_ENOMEM. */
+int ising_selftest_alloc_limit(ising_ctx* ctx, int64_t bytes);
 
 /* ------------------------------------------------------------------ energy */
 

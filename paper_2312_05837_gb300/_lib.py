@@ -113,6 +113,7 @@ _PROTOS = {
     "ising_ds_work": (c_int, [c_void_p, POINTER(c_int64)]),
     "ising_ds_set_tiles": (c_int, [c_void_p, c_int32, c_int32]),
     "ising_selftest_waits": (c_int, [c_void_p, c_int64, c_void_p]),
+    "ising_selftest_alloc_limit": (c_int, [c_void_p, c_int64]),
     "ising_ds_result": (c_int, [c_void_p, c_void_p, POINTER(c_double), POINTER(DSStats), c_int]),
     "ising_ds_destroy": (c_int, [c_void_p]),
     "ising_pack_create": (c_int, [c_void_p, POINTER(c_void_p), c_int32, POINTER(c_void_p)]),

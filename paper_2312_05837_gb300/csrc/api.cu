@@ -186,6 +186,13 @@ extern "C" int ising_selftest_waits(ising_ctx* ctx, int64_t limit_cycles, int32_
   return ISING_OK;
 }
 
+extern "C" int ising_selftest_alloc_limit(ising_ctx* ctx, int64_t bytes) {
+  if (!ctx) return ISING_EINVAL;
+  if (bytes < 0) return fail(ctx, ISING_EINVAL, "bytes must be >= 0");
+  ctx->alloc_limit = (size_t)bytes;
+  return ISING_OK;
+}
+
 namespace ising {
 int prune_device(ising_ctx* ctx, const DevInstance& I, int flags, ising_prune_result** out);
 int ds_create_impl(ising_ctx* ctx, const ising_instance* inst, const ising_ds_params* p,

@@ -19,6 +19,7 @@ struct ising_ctx {
   cudaStream_t stream = nullptr;
   int sm_count = 0;
   size_t smem_optin = 0;
+  size_t alloc_limit = 0;  // largest device allocation (0: any), for tests
   std::string err;
 };
 
@@ -105,6 +106,8 @@ inline int dev_alloc(ising_ctx* ctx, DevMem& m, size_t bytes) {
   m.release();
   if (bytes == 0) bytes = 16;
   m.stream = ctx->stream;
+  if (ctx->alloc_limit && bytes > ctx->alloc_limit)
+    return fail(ctx, ISING_ENOMEM, "device allocation of %zu bytes exceeds the limit set", bytes);
   cudaError_t e = cudaMallocAsync(&m.p, bytes, m.stream);
   if (e != cudaSuccess) {
     m.p = nullptr;

@@ -763,15 +763,17 @@ int energy_device(ising_ctx* ctx, const DevInstance& inst, const int8_t* spins, 
   const bool exact = inst.j_integer && inst.j_absmax < 2147483648.0 && inst.h_dyadic;
   if (count > 65535) return fail(ctx, ISING_EINVAL, "energy: count > 65535 per call");
   bool ok = false;
-  int shift = 0, splits = 1;
+  int shift = 0, splits = 1, rc = ISING_OK;
   if (inst.layout == ISING_LAYOUT_DENSE) {
     const double terms = (double)inst.n * (double)inst.n * (double)count;
     if (!(exact && terms < 2097152.0) && fixed_scale(inst, &shift, &splits))
-      ISING_TRY(energy_fixed(ctx, inst, exact, shift, splits, spins, count, E, Q, H, &ok));
+      rc = energy_fixed(ctx, inst, exact, shift, splits, spins, count, E, Q, H, &ok);
   } else if (packed_pays(inst, exact, count)) {
-    ISING_TRY(energy_packed(ctx, inst, exact, spins, count, E, Q, H, &ok));
+    rc = energy_packed(ctx, inst, exact, spins, count, E, Q, H, &ok);
   }
-  return ok ? ISING_OK : energy_general(ctx, inst, exact, spins, count, E, Q, H);
+  // (no room for a form's scratch: the general form's is smaller)
+  if (rc != ISING_OK && rc != ISING_ENOMEM) return rc;
+  return rc == ISING_OK && ok ? ISING_OK : energy_general(ctx, inst, exact, spins, count, E, Q, H);
 }
 
 }  // namespace ising
