@@ -611,12 +611,20 @@ int sr_launch_pack(ising_ds* ds, const SparseRes* R, const SrArgs& a) {
 
 }  // namespace
 
+static int sparse_res_layout(ising_ds* ds);
+
 // Whether the session runs this form, and its operands. It does when the
 // state of RB restarts fits a CTA's shared memory (n RB up to about 16300,
 // 14300 with 16-bit spins), with RB the least of 1, 2, 4, 8 that gives every SM at most one CTA, or 8
 // (several waves of CTAs then): the launch-per-step form costs at least two
 // launches and an L2 round trip per coupling however small the instance.
+// Where the operands find no room, the session takes a launch per step.
 int sparse_res_setup(ising_ds* ds) {
+  const int rc = sparse_res_layout(ds);
+  return rc == ISING_ENOMEM ? ISING_OK : rc;
+}
+
+static int sparse_res_layout(ising_ds* ds) {
   ising_ctx* ctx = ds->ctx;
   if ((ds->p.flags & ISING_DS_STREAMING) || ds->relaxed()) return ISING_OK;
   const DevInstance& I = ds->inst;

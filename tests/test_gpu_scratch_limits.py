@@ -63,3 +63,23 @@ def test_digit_planes(gpu_ctx):
     with _limit(gpu_ctx, 6 * n * n):  # the instance, and not its planes
         E = api.energy(gpu_ctx, _device(inst), torch.as_tensor(s).cuda())
     np.testing.assert_allclose(E.cpu().numpy(), ref, rtol=1e-12, atol=1e-9)
+
+
+def test_sparse_session_without_room_for_its_slices(gpu_ctx):
+    """FP32 couplings: 4 bytes each in every list but the slices (8 and padding)."""
+    inst = synth.random_sparse_instance(900, 4, p=0.2, kind="float", h="zero")
+    inst.data = inst.data.astype(np.float32)
+    nnz = len(inst.data)
+    kw = dict(restarts=3, steps=12, seed=5)
+    with _limit(gpu_ctx, 6 * nnz):
+        s = api.Session(gpu_ctx, inst, **kw)
+        s.run(12)
+        a, fa = s.restart_best(), s.result()["resident"]
+        s.close()
+    s = api.Session(gpu_ctx, inst, **kw)
+    s.run(12)
+    b, fb = s.restart_best(), s.result()["resident"]
+    s.close()
+    assert (fa, fb) == (0, 3)
+    for x, y in zip(a, b):
+        np.testing.assert_array_equal(x, y)
