@@ -392,6 +392,8 @@ int fixed_launch_t(ising_ctx* ctx, const DevInstance& I, int shift, int splits, 
 // products where the fixed form spends 7 integer instructions per coupling and
 // vector. Bound by writing and reading the planes (10 bytes per coupling).
 
+constexpr double kPlaneTerms = 268435456.0;  // coupling-vectors from which the form pays
+
 // Digits of every coupling, and the spins as FP16 +-1.
 template <typename T>
 __global__ void __launch_bounds__(256) split_digits_kernel(const T* __restrict__ J, int64_t n, int64_t ld,
@@ -681,7 +683,7 @@ int energy_fixed(ising_ctx* ctx, const DevInstance& inst, bool exact, int shift,
   int w = 0, planes = 0, pshift = 0, rc = ISING_ENOMEM;  // (or no room for the planes)
   // (from 16 vectors and 2^28 coupling-vectors on: n = 4096 takes 35 us per four
   // vectors in the fixed form and about 200 us for 256 in planes)
-  if (count >= 16 && (double)n * (double)n * (double)count >= 268435456.0 &&
+  if (count >= 16 && (double)n * (double)n * (double)count >= kPlaneTerms &&
       plane_scale(inst, &w, &planes, &pshift))
     rc = plane_limbs(ctx, inst, w, planes, pshift, spins, count, L);
   if (rc == ISING_OK) shift = pshift;
@@ -740,11 +742,22 @@ int energy_packed(ising_ctx* ctx, const DevInstance& inst, bool exact, const int
 
 // Which form runs: the fixed form for every dense J that one scale holds (at
 // n = 4096 FP32: 256 vectors 23.5 ms in the general form, 2.5 in the fixed, 0.2
-// in planes; one vector of n = 1000: 166 -> 6.4 us;
-// but small integer ones, whose general form takes fewer launches: n = 121, 51
-// vectors 99 against 109 us per call), the packed form for CSR instances where
+// in planes; one vector of n = 1000: 166 -> 6.4 us) but integers where the general
+// form is faster (few_integers), the packed form for CSR instances where
 // packed_pays, the general form otherwise and whenever a spin is not +-1.
 //
+// Integer dense J: the general form has two launches and a host read less (about
+// 10 us) and adds in 64-bit integers without FP64, but a warp walks a row of n
+// (65 ns per 1000 columns and row: 65 n us in all, n in thousands); a row and
+// vector costs it 0.1 + 0.8 n ns and the fixed form 0.45 + 0.25 n. us per call,
+// general / fixed, int8: n = 128, 16, 300 and 4000 vectors 102 / 109, 103 / 130,
+// 188 / 364; n = 256: 106 / 107, 132 / 153, 361 / 629; n = 512, 16, 300 and 1000:
+// 125 / 114, 194 / 203, 344 / 398; n = 1000, 1 and 64: 158 / 115, 217 / 158.
+bool few_integers(const DevInstance& I, int64_t count) {
+  const double n = (double)I.n, c = (double)count;
+  return n * c * (0.35 - 0.55e-3 * n) > 65.0 * n - 10000.0 && (count < 16 || n * n * c < kPlaneTerms);
+}
+
 // The packed form: a launch and a host read more (about 25 us a call), and a
 // warp walks a row alone, but a row of 32 vectors costs one warp instead of 32
 // (0.15 ns each with integers, 0.55 in FP64). us per call, general / packed, n
@@ -765,8 +778,7 @@ int energy_device(ising_ctx* ctx, const DevInstance& inst, const int8_t* spins, 
   bool ok = false;
   int shift = 0, splits = 1, rc = ISING_OK;
   if (inst.layout == ISING_LAYOUT_DENSE) {
-    const double terms = (double)inst.n * (double)inst.n * (double)count;
-    if (!(exact && terms < 2097152.0) && fixed_scale(inst, &shift, &splits))
+    if (!(exact && few_integers(inst, count)) && fixed_scale(inst, &shift, &splits))
       rc = energy_fixed(ctx, inst, exact, shift, splits, spins, count, E, Q, H, &ok);
   } else if (packed_pays(inst, exact, count)) {
     rc = energy_packed(ctx, inst, exact, spins, count, E, Q, H, &ok);
