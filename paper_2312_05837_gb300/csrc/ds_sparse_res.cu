@@ -677,6 +677,19 @@ static int sparse_res_layout(ising_ds* ds) {
   R.entries = (int64_t)info[0] * 32;
   // two restarts' neighbour sums share a word, 16 bits each
   if (v8 && R.rb > 1 && I.j_absmax * (double)info[1] >= 32768.0) return ISING_OK;
+  // One restart per CTA walks all couplings on as many SMs as there are restarts,
+  // 0.07 ns a slot (0.085 with 8-byte slots), where the launch-per-step form
+  // spreads its rows over the whole chip. us per step, that form / this one, with
+  // the slots: int8, 8 restarts, 312000 27.4 / 26.7, 486000 33.1 / 40.4; 152
+  // restarts 1090000 83.9 / 82.8, 1700000 111 / 127; FP32, 8 restarts, 163000 20.8 /
+  // 19.9, 277000 25.5 / 28.2, 4700000 182 / 379; 152 restarts 450000 44.0 / 40.6,
+  // 900000 68.7 / 82.9. With two or more restarts per CTA it was never the slower.
+  if (R.rb == 1 && R.entries > (v8 ? 250000 + 6000 * ds->B : 150000 + 2600 * ds->B)) return ISING_OK;
+  // FP32 energies keep the other form's rows per block: with very many restarts
+  // under the convergence rule a CTA has a warp or two and each thread many rows
+  // (300 spins of degree 48, 16384 restarts: 45 ms a run against 10; degree 12,
+  // 170 slots a thread: 20 against 47 or, where all stop early, 6.6 against 5.2)
+  if (R.entries > 6 * (int64_t)R.nt * R.nt) return ISING_OK;
   // a few long rows would pad their slices and leave the other lanes idle
   if (R.entries > 6 * nnz + 32768) return ISING_OK;
   ISING_TRY(dev_alloc(ctx, R.ell, (size_t)R.entries * ebytes));

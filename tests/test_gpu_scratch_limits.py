@@ -67,7 +67,7 @@ def test_digit_planes(gpu_ctx):
 
 def test_sparse_session_without_room_for_its_slices(gpu_ctx):
     """FP32 couplings: 4 bytes each in every list but the slices (8 and padding)."""
-    inst = synth.random_sparse_instance(900, 4, p=0.2, kind="float", h="zero")
+    inst = synth.random_sparse_instance(900, 4, p=0.12, kind="float", h="zero")
     inst.data = inst.data.astype(np.float32)
     nnz = len(inst.data)
     kw = dict(restarts=3, steps=12, seed=5)

@@ -47,11 +47,11 @@ def _case(name):
     if name == "fp8_rows":
         return synth.er_dense(1930, 1, mean_degree=8, weights="pm1"), dict(restarts=30000, steps=3)
     if name == "sparse_slices":
-        return (synth.random_sparse_instance(4000, 2, p=0.08, kind="float", h="zero"),
-                dict(restarts=2, steps=20))
+        return (synth.random_sparse_instance(2000, 2, p=0.15, kind="float", h="zero"),
+                dict(restarts=200, steps=20))
     if name == "sparse_int8":
         return (synth.random_sparse_instance(2000, 2, p=0.2, kind="int", h="zero", jmax=1),
-                dict(restarts=2, steps=20))
+                dict(restarts=200, steps=20))
     return _ferromagnet(2500), dict(restarts=64, steps=60, lr=1.0, precision="tc")
 
 

@@ -34,8 +34,8 @@ def _run(ctx, inst, B, T, **kw):
 
 # spins as words fit up to about 14300 / restarts per CTA, as bits up to 16300;
 # couplings stay in device memory where the state leaves no room for them
-_BOTH = [(200, 1, 3), (9000, 8, 3), (14500, 1, 2), (14800, 3, 1), (7200, 2, 200), (7800, 6, 160)]
-_INT = [(16300, 3, 1), (3300, 12, 500), (3640, 2, 400), (1800, 4, 1300)]
+_BOTH = [(200, 1, 3), (9000, 6, 3), (14500, 1, 2), (14800, 3, 1), (7200, 2, 200), (7800, 6, 160)]
+_INT = [(16300, 3, 1), (3300, 12, 500), (3640, 2, 400), (1800, 4, 1300), (2000, 140, 152)]
 
 
 @pytest.mark.parametrize("kind,n,extra,B", [(k, *c) for c in _BOTH for k in ("int", "float")] +
@@ -54,9 +54,11 @@ def test_resident_variants(gpu_ctx, kind, n, extra, B):
 
 
 # instances that the form declines: too many spins for shared memory, more
-# sites and restarts per thread than a word has bits, a row that would pad its
+# sites and restarts per thread than a word has bits, couplings that few restarts'
+# CTAs would walk too long, threads with many rows each, a row that would pad its
 # slice far beyond the others, the relaxed product
-@pytest.mark.parametrize("case", ["large", "large_float", "bits", "hub", "relaxed"])
+@pytest.mark.parametrize("case", ["large", "large_float", "bits", "few", "few_float", "rows", "hub",
+                                  "relaxed"])
 def test_declined(gpu_ctx, case):
     kw, B = {}, 4
     if case == "large":
@@ -65,6 +67,12 @@ def test_declined(gpu_ctx, case):
         inst, B = _ring(16500, "float", 3), 1
     elif case == "bits":
         inst, B = _ring(3300, "float", 12), 500
+    elif case == "few":
+        inst, B = _ring(2000, "int", 140), 8
+    elif case == "few_float":
+        inst, B = _ring(9000, "float", 12), 8
+    elif case == "rows":
+        inst, B, kw = _ring(300, "float", 23), 16384, dict(converge=True)
     elif case == "hub":
         n = 6000
         e = np.stack([np.zeros(n - 1, np.int64), np.arange(1, n)], 1)
