@@ -7,16 +7,19 @@
 // rounded spins from Sr, writes x_{t+1} and leaves the energies to a
 // kModeEnergy pass.
 //
-// Bound by FP32 issue: n B n multiply-adds, each output's in order of k (the
-// sums must not depend on the tiling). A thread holds 8 rows x 4 restarts: 32
-// multiply-adds for three shared-memory loads. J is symmetric, so the block's
-// 128 columns of row k, which are contiguous, stand for its 128 rows of column
-// k: the J tile is copied asynchronously without turning it over, three chunks
-// of 16 k deep. TN is the width that fills the SMs' waves best: at n = 1500 and
-// 512 restarts, 132 tiles of 48 (one per SM) instead of 48 tiles of 128.
-// Measured there: 279 us per step with 128 x 128 tiles loaded and used in turn,
-// 105 us now; pairs of rows by fma.rn.f32x2 take their second operand twice
-// from shared memory and are bound by it (110 us, 4 x 4 or 8 x 4 per thread).
+// n B n multiply-adds, each output's in order of k (the sums must not depend on
+// the tiling). A thread holds 8 rows x 4 restarts: 32 multiply-adds for three
+// shared-memory loads. J is symmetric, so the block's 128 columns of row k, which
+// are contiguous, stand for its 128 rows of column k: the J tile is copied
+// asynchronously without turning it over, three chunks of 16 k deep. TN is the
+// width that fills the SMs' waves best: at n = 1500 and 512 restarts, 132 tiles of
+// 48 (one per SM) instead of 48 tiles of 128. Measured there: 279 us per step with
+// 128 x 128 tiles loaded and used in turn, 102 us now.
+// What bounds it there: few warps. A tile of 48 has six, so two of an SM's four
+// schedulers hold two and two hold one; the schedulers issue in half of their
+// cycles, the FMA pipe is 38 % and the shared-memory pipe 47 % busy, DRAM 3 %
+// (ncu). Pairs of rows by fma.rn.f32x2 take their second operand twice from
+// shared memory and were slower (110 us, 4 x 4 or 8 x 4 per thread).
 #include "ds_internal.cuh"
 
 namespace ising {

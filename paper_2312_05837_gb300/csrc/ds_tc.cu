@@ -1162,7 +1162,7 @@ struct TcResArgs {
 // Energies of restarts [b0, b0 + 32) of the step in slot ps, one warp: lane k
 // returns that of restart b0 + k (b0 + k < b1). The sums are track_kernel's:
 // lane l adds rows l, l + 32, ... starting from 0, then an xor tree over the
-// lanes. Below 32 rows (at most 7 row tiles, so slices of 10 to 32 restarts) a
+// lanes. Below 32 rows (at most 7 row tiles, so slices of 3 to 64 restarts) a
 // lane forms its own restart's sum, all its row loads in flight at once; with
 // more rows and slices of at most 8 restarts the rows go to the lanes,
 // kTrackCols restarts at a time. Either way the warp waits for about one L2
