@@ -193,7 +193,9 @@ def launches_per_solve(T: int, rounds: int, path: int, resident: bool, rowsum: b
     for the last step; else step + track per step, plus the copy of improved
     bit-packed spins on the sparse path, which the next step's tracking
     launch makes when `deferred`: above 4096 spins), finish (energy-only step
-    + track (+ copy) + argmin), reconstruction (1), full-instance energy (2)."""
+    + track (+ copy) + argmin), reconstruction (1), full-instance energy (3
+    dense: spins to bits, sums, finish; 2 CSR). Not counted: uploads of small
+    tables and the candidates' energies of non-integer instances."""
     per_step = 3 if path == 2 else 2
     if resident:
         steps = 4 if path == 2 else 1
@@ -202,7 +204,7 @@ def launches_per_solve(T: int, rounds: int, path: int, resident: bool, rowsum: b
     else:
         steps = (2 * T + 1 if T else 0) if deferred else per_step * T
     setup = 4 + (1 if rowsum else 0) + (1 if rowscale else 0)
-    return 3 + 3 + 7 * (rounds + 1) + 3 + setup + steps + per_step + 1 + 1 + 2
+    return 3 + 3 + 7 * (rounds + 1) + 3 + setup + steps + per_step + 1 + 1 + (2 if path == 2 else 3)
 
 
 # ----------------------------------------------------------------- reference arm

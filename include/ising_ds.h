@@ -130,9 +130,9 @@ typedef struct ising_ds_params {
  * per step) even when a resident form would fit. The resident form of the
  * sparse path runs a whole run of steps in one launch with the state of each
  * block's restarts in shared memory (instances whose spins, state and one to
- * eight restarts fit there). The tensor-core path's resident forms keep theta,
- * m and v in tensor memory across a whole run in
- * one launch: for n <= 128 the small form (every CTA holds all of J and the
+ * eight restarts fit there; not few restarts of many couplings, whose rows all
+ * SMs share in the other form). The tensor-core path's resident forms keep
+ * theta, m and v in tensor memory across a whole run in one launch: for n <= 128 the small form (every CTA holds all of J and the
  * spins of its block of 16 to 128 restarts in shared memory, no grid-wide
  * barrier), for larger n the grid-wide form (one cooperative launch), used
  * when every tile of 128 spins and 16 to 128 restarts gets its own SM. */
